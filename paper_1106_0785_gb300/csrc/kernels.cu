@@ -193,19 +193,60 @@ void launch_inflow(R* f, const Layout& L, const Coef<R>& c, const Walls& w, cuda
 }
 
 // ---------------------------------------------------------------------------
-// Dense [16][ny][nx] <-> padded layout.
+// Dense [16][ny][nx] <-> padded layout.  A copy: 2 x the state's bytes.  The
+// rows of all planes are numbered through (q ny + j); a block takes the same
+// columns of kPackRows x blockDim.y of them, every load of a thread before its
+// first store, V values to a load (16 bytes where the dense rows allow it,
+// else one), and as many threads to a row as it fills.  4096 x 1024 in FP32 on
+// GB300, mrtlb_set_f with its other launches: 221 -> 106 us (a value per thread
+// and a block per piece of a row before); 1501 x 701, rows off the 16-byte
+// grid: 80 -> 64 us.
 // ---------------------------------------------------------------------------
+constexpr int kPackThreads = 256, kPackRows = 4;
+template <typename R, int V>
+struct alignas(sizeof(R) * V) PackVec {
+  R v[V];
+};
+template <typename R, int V>
+__global__ void __launch_bounds__(kPackThreads) pack_kernel(const R* __restrict__ from, R* __restrict__ to, Layout L,
+                                                            int to_padded) {
+  using T = PackVec<R, V>;
+  for (long long i = ((long long)blockIdx.y * blockDim.x + threadIdx.x) * V; i < L.nx;
+       i += (long long)gridDim.y * blockDim.x * V) {
+    long long src[kPackRows], dst[kPackRows];
+    T x[kPackRows];
+#pragma unroll
+    for (int k = 0; k < kPackRows; ++k) {
+      const int row = (blockIdx.x * kPackRows + k) * blockDim.y + threadIdx.y;  // q ny + j
+      if (row >= 16 * L.ny) {
+        src[k] = -1;
+        continue;
+      }
+      const int q = row / L.ny, j = row - q * L.ny;
+      const long long dense = (long long)row * L.nx + i, padded = q * L.plane + L.node(0, j) + i;
+      src[k] = to_padded ? dense : padded;
+      dst[k] = to_padded ? padded : dense;
+      x[k] = *reinterpret_cast<const T*>(from + src[k]);
+    }
+#pragma unroll
+    for (int k = 0; k < kPackRows; ++k)
+      if (src[k] >= 0) *reinterpret_cast<T*>(to + dst[k]) = x[k];
+  }
+}
+
 template <typename R>
-__global__ void pack_kernel(const R* __restrict__ dense, R* __restrict__ padded, Layout L, int to_padded) {
-  // grid: x over columns, y over rows, z over planes (no divisions)
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  const int j = blockIdx.y;
-  const int q = blockIdx.z;
-  if (i >= L.nx) return;
-  const long long d = ((long long)q * L.ny + j) * L.nx + i;
-  const long long p = q * L.plane + L.node(i, j);
-  if (to_padded) padded[p] = dense[d];
-  else ((R*)dense)[d] = padded[p];
+static void launch_copy(const R* from, R* to, const R* dense, const Layout& L, int to_padded, cudaStream_t st) {
+  constexpr int V = 16 / (int)sizeof(R);
+  const bool wide = L.nx % V == 0 && ((uintptr_t)dense & 15) == 0;  // (padded rows start on 128 bytes)
+  const int per_row = wide ? L.nx / V : L.nx;
+  int bx = 1;
+  while (bx < kPackThreads && bx < per_row) bx *= 2;
+  const dim3 blk(bx, kPackThreads / bx);
+  const int rows = kPackRows * (int)blk.y;
+  const int pieces = (per_row - 1) / bx + 1;
+  const dim3 grd((16 * L.ny + rows - 1) / rows, pieces < 65535 ? pieces : 65535);
+  if (wide) pack_kernel<R, V><<<grd, blk, 0, st>>>(from, to, L, to_padded);
+  else pack_kernel<R, 1><<<grd, blk, 0, st>>>(from, to, L, to_padded);
 }
 
 static int grid_for(long long n, int threads) {
@@ -217,13 +258,11 @@ static int grid_for(long long n, int threads) {
 
 template <typename R>
 void launch_pack(const R* dense, R* padded, const Layout& L, cudaStream_t st) {
-  dim3 grd((L.nx + 255) / 256, L.ny, 16);
-  pack_kernel<R><<<grd, 256, 0, st>>>(dense, padded, L, 1);
+  launch_copy<R>(dense, padded, dense, L, 1, st);
 }
 template <typename R>
 void launch_unpack(const R* padded, R* dense, const Layout& L, cudaStream_t st) {
-  dim3 grd((L.nx + 255) / 256, L.ny, 16);
-  pack_kernel<R><<<grd, 256, 0, st>>>(dense, (R*)padded, L, 0);
+  launch_copy<R>(padded, dense, dense, L, 0, st);
 }
 
 // ---------------------------------------------------------------------------
