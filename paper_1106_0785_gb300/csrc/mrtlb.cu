@@ -415,6 +415,14 @@ static void enqueue_bc(mrtlb_ctx* c, void* f) {
   }
 }
 
+// Wall nodes (and diffuse ghosts) that follow their neighbours: all that a
+// step or a read of f needs, since the steps keep the other ghosts complete
+// and a read does not look at them.
+static void enqueue_walls(mrtlb_ctx* c, void* f, cudaStream_t st) {
+  if (c->prec == MRTLB_FP64) launch_walls<double>((double*)f, c->L, c->c64, c->walls, st);
+  else launch_walls<float>((float*)f, c->L, c->c32, c->walls, st);
+}
+
 static int check_launch(mrtlb_ctx* c, const char* what) {
   const cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return cuda_fail(c, e, what);
@@ -455,8 +463,7 @@ static void enqueue_one(mrtlb_ctx* c, int cur, cudaStream_t st, bool timed) {
   void* fin = c->f[cur];
   void* fout = c->f[cur ^ 1];
   // (ghosts of fin were written through by the previous step)
-  if (c->prec == MRTLB_FP64) launch_walls<double>((double*)fin, c->L, c->c64, c->walls, st);
-  else launch_walls<float>((float*)fin, c->L, c->c32, c->walls, st);
+  enqueue_walls(c, fin, st);
   if (timed) cudaEventRecord(c->ev[2 * c->ev_used], st);
   if (c->prec == MRTLB_FP64) {
     if (tiled) launch_step_tiled<double>(c->plan, cur, c->L, c->c64, c->err, st, fout);
@@ -561,7 +568,7 @@ extern "C" int mrtlb_macros(mrtlb_ctx* c, double* rho, double* ux, double* uy, d
   if (!bound(c)) return c ? fail(c, MRTLB_ERR_STATE, "bind state buffers first") : MRTLB_ERR_ARG;
   const size_t n = (size_t)c->L.nx * c->L.ny;
   void* f = c->f[c->cur];
-  enqueue_bc(c, f);  // wall nodes follow the current neighbours
+  enqueue_walls(c, f, c->stream);
   double* d[4] = {rho, ux, uy, T};
   double* dd[4] = {rho, ux, uy, T};
   bool direct = !on_device;
@@ -591,7 +598,7 @@ extern "C" int mrtlb_reduce(mrtlb_ctx* c, double out[5]) {
   const size_t n = (size_t)c->L.nx * c->L.ny;
   if (!c->Tprev) CK(cudaMalloc((void**)&c->Tprev, n * sizeof(double)), "cudaMalloc(Tprev)");
   void* f = c->f[c->cur];
-  enqueue_bc(c, f);
+  enqueue_walls(c, f, c->stream);
   CK(cudaMemsetAsync(c->acc, 0, 5 * sizeof(double), c->stream), "cudaMemsetAsync");
   if (c->prec == MRTLB_FP64) launch_reduce<double>((const double*)f, c->acc, c->Tprev, c->have_prev, c->L, c->stream);
   else launch_reduce<float>((const float*)f, c->acc, c->Tprev, c->have_prev, c->L, c->stream);
@@ -611,7 +618,7 @@ extern "C" int mrtlb_get_f(mrtlb_ctx* c, void* f, int on_device) {
   if (!f) return fail(c, MRTLB_ERR_ARG, "f is NULL");
   const size_t bytes = (size_t)16 * c->L.nx * c->L.ny * c->esize;
   void* cur = c->f[c->cur];
-  enqueue_bc(c, cur);
+  enqueue_walls(c, cur, c->stream);
   void* dst = f;
   void* direct = on_device ? nullptr : mapped_host(f);
   if (direct) {
