@@ -243,6 +243,13 @@ int plan_tiled(const Layout& L, int esize, void* f0, void* f1, TiledPlan* plan) 
       }
     }
   }
+  // The CTAs with which a march of short segments (8 rows or more) beats the
+  // plain kernel, measured on GB300, us per step, plain / march: FP32 700 x 500
+  // (2.5 CTAs per SM) 13.4 / 16.7, 1501 x 300 (3.0) 16.5 / 15.4, 1000 x 600
+  // (3.9) 23.1 / 16.1, 1501 x 701 (segments of 15 rows) 44.1 / 28.4; FP64
+  // 1024 x 128 (1.7) 132 / 130, 1000 x 150 (2.0) 151 / 130, 1024 x 256 (3.0)
+  // 262 / 225.
+  plan->fill = (esize == 4 ? 3 : 2) * nsm;
   plan->ok = true;
   return 0;
 }
@@ -275,8 +282,9 @@ bool use_tiled(int which, const TiledPlan& plan, bool fp64) {
   if (which == MRTLB_KERNEL_PLAIN) return false;
   if (which == MRTLB_KERNEL_TILED) return true;
   // AUTO: a march of a few rows is latency-bound (each row waits for its
-  // copy); small grids go to the one-thread-per-node kernel
-  return plan.seglen >= kMinMarchRows;
+  // copy) unless there are enough of them to fill the device; smaller grids
+  // go to the one-thread-per-node kernel
+  return plan.seglen >= kMinMarchRows || plan.nstrips * plan.nseg >= plan.fill;
 }
 
 template <typename R>
