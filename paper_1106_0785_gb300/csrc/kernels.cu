@@ -6,29 +6,29 @@ namespace mrtlb {
 
 // ---------------------------------------------------------------------------
 // Plain step: one thread per advanced node, neighbours read straight from
-// global memory (L1/L2 serve the reuse).  Used for the FP64 path and as the
-// reference launch shape for the FP32 path.
+// global memory (L1/L2 serve the reuse).  The choice for grids too small for
+// the row march, and the reference for it.
+//
+// REFILL: walls and diffuse ghosts are functions of the node beside them, so
+// the node works them out from its own distributions and a step needs no
+// launch before it that refills them in memory (whoever reads them there
+// refills them first).
 // ---------------------------------------------------------------------------
 template <typename R>
-__device__ __forceinline__ void node_velocity(const R* __restrict__ f, long long plane, long long at,
-                                              R& ux, R& uy) {
-  R g[16];
-#pragma unroll
-  for (int q = 0; q < 16; ++q) g[q] = f[q * plane + at];
+__device__ __forceinline__ void velocity(const R g[16], R& ux, R& uy) {
   R rho, jx, jy, e;
   conserved(g, rho, jx, jy, e);
   const R r = recip(rho);
   ux = jx * r;
   uy = jy * r;
 }
-
 // Thread t takes advanced node t of the row-major enumeration of
 // [i0, i1) x [j0, j1), so that every lane of a warp has a node whatever the
 // grid's shape (a 4-column grid would leave 28 of 32 lanes idle under a
 // 2D block, and FP64 arithmetic costs a warp the same with idle lanes).
-template <typename R>
+template <typename R, bool REFILL>
 __global__ void __launch_bounds__(128) step_plain_kernel(const R* __restrict__ fin, R* __restrict__ fout,
-                                                         Layout L, Coef<R> c, int* err) {
+                                                         Layout L, Coef<R> c, Walls w, int* err) {
   const int ni = L.i1 - L.i0;
   const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= (long long)ni * (L.j1 - L.j0)) return;
@@ -47,13 +47,20 @@ __global__ void __launch_bounds__(128) step_plain_kernel(const R* __restrict__ f
   const R ux = jx * ir, uy = jy * ir;
   const R T = temperature(rho, jx, jy, e, ir);
 
-  R uxE, uyE, uxW, uyW, uxN, uyN, uxS, uyS;
-  node_velocity(fin, P, E, uxE, uyE);
-  node_velocity(fin, P, W, uxW, uyW);
-  node_velocity(fin, P, N, uxN, uyN);
-  node_velocity(fin, P, S, uxS, uyS);
-  const R dux_dx = (uxE - uxW) * c.inv2dx, duy_dx = (uyE - uyW) * c.inv2dx;
-  const R dux_dy = (uxN - uxS) * c.inv2dy, duy_dy = (uyN - uyS) * c.inv2dy;
+  R uxn[4], uyn[4], b[4][16];  // beyond sides -x, +x, -y, +y
+  const long long nb[4] = {W, E, S, N};
+#pragma unroll
+  for (int s = 0; s < 4; ++s) {
+    if (REFILL && beside_refilled(L, s, i, j)) {
+      refilled_value(c, w, L, s, f, b[s]);
+    } else {
+#pragma unroll
+      for (int q = 0; q < 16; ++q) b[s][q] = fin[q * P + nb[s]];
+    }
+    velocity(b[s], uxn[s], uyn[s]);
+  }
+  const R dux_dx = (uxn[1] - uxn[0]) * c.inv2dx, duy_dx = (uyn[1] - uyn[0]) * c.inv2dx;
+  const R dux_dy = (uxn[3] - uxn[2]) * c.inv2dy, duy_dy = (uyn[3] - uyn[2]) * c.inv2dy;
 
   R C[16];
   collision(c, f, dux_dx, dux_dy, duy_dx, duy_dy, rho, ir, jx, jy, e, ux, uy, T, C);
@@ -61,8 +68,9 @@ __global__ void __launch_bounds__(128) step_plain_kernel(const R* __restrict__ f
   R vout[16];
 #pragma unroll
   for (int q = 0; q < 16; ++q) {
-    const R fE = (vx_of(q) != 0) ? fin[q * P + E] : R(0), fW = (vx_of(q) != 0) ? fin[q * P + W] : R(0);
-    const R fN = (vy_of(q) != 0) ? fin[q * P + N] : R(0), fS = (vy_of(q) != 0) ? fin[q * P + S] : R(0);
+    // (without REFILL read again, from L1, instead of held in registers)
+    const R fE = REFILL ? b[1][q] : fin[q * P + E], fW = REFILL ? b[0][q] : fin[q * P + W];
+    const R fN = REFILL ? b[3][q] : fin[q * P + N], fS = REFILL ? b[2][q] : fin[q * P + S];
     const R fn = lw_update(c, q, f[q], C[q], fE, fW, fN, fS);
     fout[q * P + at] = fn;
     vout[q] = fn;
@@ -73,7 +81,7 @@ __global__ void __launch_bounds__(128) step_plain_kernel(const R* __restrict__ f
 }
 
 template <typename R>
-void launch_step_plain(const R* fin, R* fout, const Layout& L, const Coef<R>& c, int* err,
+void launch_step_plain(const R* fin, R* fout, const Layout& L, const Coef<R>& c, const Walls* w, int* err,
                        cudaStream_t st) {
   const int ni = L.i1 - L.i0, nj = L.j1 - L.j0;
   if (ni <= 0 || nj <= 0) return;
@@ -89,7 +97,10 @@ void launch_step_plain(const R* fin, R* fout, const Layout& L, const Coef<R>& c,
   const long long n = (long long)ni * nj;
   int blk = 8;
   while (blk < 128 && (long long)blk * nsm < n) blk *= 2;
-  step_plain_kernel<R><<<(unsigned)((n + blk - 1) / blk), blk, 0, st>>>(fin, fout, L, c, err);
+  const unsigned grd = (unsigned)((n + blk - 1) / blk);
+  const bool refill = w && wall_count(L) > 0;
+  if (refill) step_plain_kernel<R, true><<<grd, blk, 0, st>>>(fin, fout, L, c, *w, err);
+  else step_plain_kernel<R, false><<<grd, blk, 0, st>>>(fin, fout, L, c, Walls{}, err);
 }
 
 // ---------------------------------------------------------------------------
@@ -103,24 +114,12 @@ __global__ void bc_walls_kernel(R* f, Layout L, Coef<R> c, Walls w) {
   wall_node(f, L, c, w, blockIdx.x * blockDim.x + threadIdx.x);
 }
 
-// f^eq of an inflow side's fixed state, plane q.
-template <typename R>
-__device__ __forceinline__ R inflow_value(const Coef<R>& c, const Walls& w, int side, int q) {
-  const R rho = (R)w.rho[side], ux = (R)w.ux[side], uy = (R)w.uy[side], T = (R)w.T[side];
-  const R ir = R(1) / rho;
-  R eq[16], fe[16];
-  equilibrium(c, rho, ir, rho * ux, rho * uy, rho * (T + R(0.5) * (ux * ux + uy * uy)), ux, uy, T, eq);
-  inverse_full(c, eq, fe);
-  return fe[q];
-}
-
 // One ghost value beside side s of a non-periodic side from the edge node
 // `edge` (plane-0 address): outflow and walls copy it, reflect takes the
 // mirrored plane, inflow the side's fixed equilibrium.
 template <typename R>
-__device__ __forceinline__ R side_ghost(const Coef<R>& c, const Walls& w, const Layout& L, int s, int q,
-                                        const R* edge) {
-  if (L.bc[s] == BC_INFLOW) return inflow_value(c, w, s, q);
+__device__ __forceinline__ R side_ghost(const Walls& w, const Layout& L, int s, int q, const R* edge) {
+  if (L.bc[s] == BC_INFLOW) return (R)(w.rho[s] * w.e64[s][q]);
   if (L.bc[s] == BC_REFLECT) return edge[(long long)(s < 2 ? mirror_x(q) : mirror_y(q)) * L.plane];
   return edge[(long long)q * L.plane];
 }
@@ -129,7 +128,7 @@ __device__ __forceinline__ R side_ghost(const Coef<R>& c, const Walls& w, const 
 // wall pass fills those).  only_inflow: just the inflow sides (buffers whose
 // other ghosts the steps write).
 template <typename R>
-__global__ void bc_ghost_kernel(R* f, Layout L, Coef<R> c, Walls w, int only_inflow) {
+__global__ void bc_ghost_kernel(R* f, Layout L, Walls w, int only_inflow) {
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
   const int q = blockIdx.y;
   const long long P = L.plane;
@@ -145,9 +144,9 @@ __global__ void bc_ghost_kernel(R* f, Layout L, Coef<R> c, Walls w, int only_inf
       }
     } else {
       if ((!only_inflow && L.bc[0] != BC_DIFFUSE) || L.bc[0] == BC_INFLOW)
-        fq[first - 1] = side_ghost(c, w, L, 0, q, f + first);
+        fq[first - 1] = side_ghost(w, L, 0, q, f + first);
       if ((!only_inflow && L.bc[1] != BC_DIFFUSE) || L.bc[1] == BC_INFLOW)
-        fq[last + 1] = side_ghost(c, w, L, 1, q, f + last);
+        fq[last + 1] = side_ghost(w, L, 1, q, f + last);
     }
   }
   if (t < L.nx) {  // y sides, column i = t
@@ -161,9 +160,9 @@ __global__ void bc_ghost_kernel(R* f, Layout L, Coef<R> c, Walls w, int only_inf
       }
     } else {
       if ((!only_inflow && L.bc[2] != BC_DIFFUSE) || L.bc[2] == BC_INFLOW)
-        fq[first - L.pitch] = side_ghost(c, w, L, 2, q, f + first);
+        fq[first - L.pitch] = side_ghost(w, L, 2, q, f + first);
       if ((!only_inflow && L.bc[3] != BC_DIFFUSE) || L.bc[3] == BC_INFLOW)
-        fq[last + L.pitch] = side_ghost(c, w, L, 3, q, f + last);
+        fq[last + L.pitch] = side_ghost(w, L, 3, q, f + last);
     }
   }
 }
@@ -179,7 +178,7 @@ void launch_bc(R* f, const Layout& L, const Coef<R>& c, const Walls& w, cudaStre
   launch_walls<R>(f, L, c, w, st);
   const int n = (L.nx > L.ny) ? L.nx : L.ny;
   dim3 grd((n + 255) / 256, 16);
-  bc_ghost_kernel<R><<<grd, 256, 0, st>>>(f, L, c, w, 0);
+  bc_ghost_kernel<R><<<grd, 256, 0, st>>>(f, L, w, 0);
 }
 
 template <typename R>
@@ -189,7 +188,7 @@ void launch_inflow(R* f, const Layout& L, const Coef<R>& c, const Walls& w, cuda
   if (!any) return;
   const int n = (L.nx > L.ny) ? L.nx : L.ny;
   dim3 grd((n + 255) / 256, 16);
-  bc_ghost_kernel<R><<<grd, 256, 0, st>>>(f, L, c, w, 1);
+  bc_ghost_kernel<R><<<grd, 256, 0, st>>>(f, L, w, 1);
 }
 
 // ---------------------------------------------------------------------------
@@ -380,8 +379,8 @@ void launch_reduce(const R* f, double* acc, double* Tprev, int have_prev, const 
 }
 
 #define MRTLB_INSTANTIATE(R)                                                                     \
-  template void launch_step_plain<R>(const R*, R*, const Layout&, const Coef<R>&, int*,          \
-                                     cudaStream_t);                                              \
+  template void launch_step_plain<R>(const R*, R*, const Layout&, const Coef<R>&, const Walls*,   \
+                                     int*, cudaStream_t);                                        \
   template void launch_bc<R>(R*, const Layout&, const Coef<R>&, const Walls&, cudaStream_t); \
   template void launch_walls<R>(R*, const Layout&, const Coef<R>&, const Walls&, cudaStream_t); \
   template void launch_inflow<R>(R*, const Layout&, const Coef<R>&, const Walls&, cudaStream_t); \

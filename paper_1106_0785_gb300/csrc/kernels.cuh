@@ -99,7 +99,16 @@ __device__ __forceinline__ void write_ghosts(const GhostTargets& g, long long pl
 struct Walls {
   double ux[4], uy[4], T[4];  // per side: wall or inflow velocity and temperature
   double rho[4];              // inflow density
+  // Constants of the sides, worked out once on the host in FP64: the side's
+  // equilibrium distributions at unit density (walls, diffuse, inflow) in both
+  // precisions, and for a diffuse side the weights of the edge node's f_q and
+  // the divisor in its density (diffuse_value).
+  double e64[4][16];
+  float e32[4][16];
+  double num[4][16], den[4];
 };
+__device__ __forceinline__ double side_e(const Walls& w, int s, int q, double) { return w.e64[s][q]; }
+__device__ __forceinline__ float side_e(const Walls& w, int s, int q, float) { return w.e32[s][q]; }
 
 // Boundary cells refilled before every step: NEE wall nodes (ny per x side,
 // nx per y side) and diffuse-reflection ghost cells (likewise).
@@ -126,85 +135,89 @@ __device__ __forceinline__ void wall_equilibrium(const Coef<R>& c, R ux, R uy, R
 // and b_q the edge node's in the ghost position's,
 //   rho_w = (sum_q b_q f_q - sum_{q not entering} a_q f_q) / sum_{q entering} a_q e_q.
 template <typename R>
-__device__ __forceinline__ bool entering(int s, int q) {
+MRTLB_HD bool entering(int s, int q) {
   return (s == 0) ? vx_of(q) > 0 : (s == 1) ? vx_of(q) < 0 : (s == 2) ? vy_of(q) > 0 : vy_of(q) < 0;
 }
 template <typename R>
-__device__ __forceinline__ void diffuse_weights(const Coef<R>& c, int s, int q, R& a, R& b) {
+MRTLB_HD void diffuse_weights(const Coef<R>& c, int s, int q, R& a, R& b) {
   const int ga = (s == 0) ? 1 : (s == 1) ? 0 : (s == 2) ? 3 : 2;  // lw index of the ghost neighbour
   a = c.lw[q][ga];
   b = c.lw[q][ga ^ 1];
 }
+// The flux balance is in FP64 from the weights the update uses: in FP32 its
+// rounding would leak mass the same way at every step (e cancels out of the
+// balance, so its own rounding does not).
 template <typename R>
-__device__ __forceinline__ void diffuse_ghost(const Coef<R>& c, const Walls& w, const Layout& L, int s,
-                                              const R* edge, R* ghost) {
-  R e[16], f[16];
-  wall_equilibrium(c, (R)w.ux[s], (R)w.uy[s], (R)w.T[s], e);
-  // the flux balance in FP64 from the weights the update uses: in FP32 its
-  // rounding would leak mass the same way at every step (e cancels out of
-  // the balance, so its own rounding does not)
-  double num = 0.0, den = 0.0;
+__device__ __forceinline__ void diffuse_value(const Walls& w, int s, const R f[16], R ghost[16]) {
+  double num = 0.0;
 #pragma unroll
-  for (int q = 0; q < 16; ++q) {
-    f[q] = edge[(long long)q * L.plane];
-    R a, b;
-    diffuse_weights(c, s, q, a, b);
-    num += (double)b * (double)f[q];
-    if (entering<R>(s, q)) den += (double)a * (double)e[q];
-    else num -= (double)a * (double)f[q];
-  }
-  const double rw = num / den;
+  for (int q = 0; q < 16; ++q) num += w.num[s][q] * (double)f[q];
+  const double rw = num / w.den[s];
 #pragma unroll
-  for (int q = 0; q < 16; ++q)
-    ghost[(long long)q * L.plane] = entering<R>(s, q) ? (R)(rw * (double)e[q]) : f[q];
+  for (int q = 0; q < 16; ++q) ghost[q] = entering<R>(s, q) ? (R)(rw * w.e64[s][q]) : f[q];
 }
 
+// The NEE wall node on side s from its fluid neighbour's distributions g:
+// f^eq(rho, u_w, T_w) + g - f^eq(rho, u, T), the first linear in rho.
 template <typename R>
-__device__ __forceinline__ void wall_node(R* f, const Layout& L, const Coef<R>& c, const Walls& w, int k) {
-  int side = -1, i = 0, j = 0, ia = 0, ja = 0;
-  for (int s = 0; s < 4 && side < 0; ++s) {
-    const int n = (s < 2) ? L.ny : L.nx;
-    if (!refilled_side(L.bc[s])) continue;
-    if (k < n) {
-      side = s;
-      if (s == 0) { i = 0; j = k; ia = 1; ja = k; }
-      if (s == 1) { i = L.nx - 1; j = k; ia = L.nx - 2; ja = k; }
-      if (s == 2) { i = k; j = 0; ia = k; ja = 1; }
-      if (s == 3) { i = k; j = L.ny - 1; ia = k; ja = L.ny - 2; }
-    } else {
-      k -= n;
-    }
-  }
-  if (side < 0) return;
-  if (L.bc[side] == BC_DIFFUSE) {  // the ghost cell beyond edge node (i, j)
-    const long long off = (side == 0) ? -1 : (side == 1) ? 1 : (side == 2) ? -(long long)L.pitch : L.pitch;
-    diffuse_ghost(c, w, L, side, f + L.node(i, j), f + L.node(i, j) + off);
-    return;
-  }
-  const long long P = L.plane;
-  const long long a = L.node(ia, ja), at = L.node(i, j);
-  R g[16];
-#pragma unroll
-  for (int q = 0; q < 16; ++q) g[q] = f[q * P + a];
+__device__ __forceinline__ void wall_value(const Coef<R>& c, const Walls& w, int s, const R g[16], R f[16]) {
   R rho, jx, jy, e;
   conserved(g, rho, jx, jy, e);
   const R ir = R(1) / rho;
   const R ux = jx * ir, uy = jy * ir;
   const R T = temperature(rho, jx, jy, e, ir);
-  R eqa[16], eqw[16], d[16], df[16];
+  R eqa[16], fa[16];
   equilibrium(c, rho, ir, jx, jy, e, ux, uy, T, eqa);
-  const R uwx = (R)w.ux[side], uwy = (R)w.uy[side], Tw = (R)w.T[side];
-  const R ew = rho * (Tw + R(0.5) * (uwx * uwx + uwy * uwy));
-  equilibrium(c, rho, ir, rho * uwx, rho * uwy, ew, uwx, uwy, Tw, eqw);
+  inverse_full(c, eqa, fa);
 #pragma unroll
-  for (int q = 0; q < 16; ++q) d[q] = eqw[q] - eqa[q];
-  inverse_full(c, d, df);
-#pragma unroll
-  for (int q = 0; q < 16; ++q) f[q * P + at] = g[q] + df[q];
+  for (int q = 0; q < 16; ++q) f[q] = g[q] + (rho * side_e(w, s, q, R()) - fa[q]);
+}
+
+// What lies beyond advanced node (i, j) across side s when that side is
+// refilled before every step: a wall node or a diffuse ghost, either of them
+// a function of the node's own distributions.
+__device__ __forceinline__ bool beside_refilled(const Layout& L, int s, int i, int j) {
+  return refilled_side(L.bc[s]) &&
+         (s == 0 ? i == L.i0 : s == 1 ? i == L.i1 - 1 : s == 2 ? j == L.j0 : j == L.j1 - 1);
+}
+template <typename R>
+__device__ __forceinline__ void refilled_value(const Coef<R>& c, const Walls& w, const Layout& L, int s, const R g[16],
+                                               R f[16]) {
+  if (L.bc[s] == BC_WALL) wall_value(c, w, s, g, f);
+  else diffuse_value(w, s, g, f);
 }
 
 template <typename R>
-void launch_step_plain(const R* fin, R* fout, const Layout& L, const Coef<R>& c, int* err,
+__device__ __forceinline__ void wall_node(R* f, const Layout& L, const Coef<R>& c, const Walls& w, int k) {
+  int side = -1, i = 0, j = 0;
+  for (int s = 0; s < 4 && side < 0; ++s) {
+    const int n = (s < 2) ? L.ny : L.nx;
+    if (!refilled_side(L.bc[s])) continue;
+    if (k < n) {
+      side = s;
+      i = (s == 0) ? 0 : (s == 1) ? L.nx - 1 : k;
+      j = (s == 2) ? 0 : (s == 3) ? L.ny - 1 : k;
+    } else {
+      k -= n;
+    }
+  }
+  if (side < 0) return;
+  const long long P = L.plane;
+  const long long in = (side == 0) ? 1 : (side == 1) ? -1 : (side == 2) ? L.pitch : -(long long)L.pitch;
+  // a wall node follows the node inside of it, a diffuse ghost its edge node
+  const long long at = L.node(i, j) - (L.bc[side] == BC_DIFFUSE ? in : 0);
+  R g[16], v[16];
+#pragma unroll
+  for (int q = 0; q < 16; ++q) g[q] = f[q * P + at + in];
+  refilled_value(c, w, L, side, g, v);
+#pragma unroll
+  for (int q = 0; q < 16; ++q) f[q * P + at] = v[q];
+}
+
+// One step by the one-thread-per-node kernel.  With `w` it works out the walls
+// and diffuse ghosts beside its nodes itself; without, it reads them from fin.
+template <typename R>
+void launch_step_plain(const R* fin, R* fout, const Layout& L, const Coef<R>& c, const Walls* w, int* err,
                        cudaStream_t st);
 template <typename R>
 void launch_bc(R* f, const Layout& L, const Coef<R>& c, const Walls& w, cudaStream_t st);

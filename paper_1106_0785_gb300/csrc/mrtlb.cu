@@ -232,6 +232,35 @@ static int build_coefficients(mrtlb_ctx* c) {
   return MRTLB_OK;
 }
 
+// The constants of the sides that hold a state (Walls), from the weights of
+// the context's precision.
+static void build_sides(mrtlb_ctx* c) {
+  Walls& w = c->walls;
+  for (int s = 0; s < 4; ++s) {
+    const int kind = c->L.bc[s];
+    if (!refilled_side(kind) && kind != BC_INFLOW) continue;
+    double eq[16];
+    const double ux = w.ux[s], uy = w.uy[s], T = w.T[s];
+    equilibrium(c->c64, 1.0, 1.0, ux, uy, T + 0.5 * (ux * ux + uy * uy), ux, uy, T, eq);
+    inverse_full(c->c64, eq, w.e64[s]);
+    w.den[s] = 0.0;
+    for (int q = 0; q < 16; ++q) {
+      w.e32[s][q] = (float)w.e64[s][q];
+      double a, b;
+      if (c->prec == MRTLB_FP64) {
+        diffuse_weights(c->c64, s, q, a, b);
+      } else {
+        float a32, b32;
+        diffuse_weights(c->c32, s, q, a32, b32);
+        a = a32, b = b32;
+      }
+      const bool in = entering<double>(s, q);
+      w.num[s][q] = in ? b : b - a;
+      if (in) w.den[s] += a * w.e64[s][q];
+    }
+  }
+}
+
 extern "C" int mrtlb_create(const mrtlb_params* params, mrtlb_ctx** out) {
   mrtlb_ctx* c = nullptr;
   g_create_error.clear();
@@ -334,6 +363,7 @@ extern "C" int mrtlb_create(const mrtlb_params* params, mrtlb_ctx** out) {
     delete c;
     return rc;
   }
+  build_sides(c);
   *out = c;
   return MRTLB_OK;
 }
@@ -457,20 +487,20 @@ extern "C" int mrtlb_init_equilibrium(mrtlb_ctx* c, const double* rho, const dou
   return check_launch(c, "init_equilibrium");
 }
 
-// one step reading buffer `cur` (walls refilled, then the step kernel)
+// one step reading buffer `cur` (for the march the walls refilled first)
 static void enqueue_one(mrtlb_ctx* c, int cur, cudaStream_t st, bool timed) {
   const bool tiled = use_tiled(c->kernel, c->plan, c->prec == MRTLB_FP64);
   void* fin = c->f[cur];
   void* fout = c->f[cur ^ 1];
   // (ghosts of fin were written through by the previous step)
-  enqueue_walls(c, fin, st);
+  if (tiled) enqueue_walls(c, fin, st);
   if (timed) cudaEventRecord(c->ev[2 * c->ev_used], st);
   if (c->prec == MRTLB_FP64) {
     if (tiled) launch_step_tiled<double>(c->plan, cur, c->L, c->c64, c->err, st, fout);
-    else launch_step_plain<double>((const double*)fin, (double*)fout, c->L, c->c64, c->err, st);
+    else launch_step_plain<double>((const double*)fin, (double*)fout, c->L, c->c64, &c->walls, c->err, st);
   } else {
     if (tiled) launch_step_tiled<float>(c->plan, cur, c->L, c->c32, c->err, st, fout);
-    else launch_step_plain<float>((const float*)fin, (float*)fout, c->L, c->c32, c->err, st);
+    else launch_step_plain<float>((const float*)fin, (float*)fout, c->L, c->c32, &c->walls, c->err, st);
   }
   if (timed) {
     cudaEventRecord(c->ev[2 * c->ev_used + 1], st);
@@ -728,6 +758,7 @@ extern "C" int mrtlb_timing_end(mrtlb_ctx* c, double* kernel_ms, long* launches)
 extern "C" int mrtlb_launches_per_step(const mrtlb_ctx* c) {
   if (!c) return MRTLB_ERR_ARG;
   int n = 1;  // the step (it writes the ghost layer through)
+  if (!use_tiled(c->kernel, c->plan, c->prec == MRTLB_FP64)) return n;  // (and works out walls itself)
   for (int s = 0; s < 4; ++s)
     if (refilled_side(c->L.bc[s])) { ++n; break; }  // + the wall and diffuse-ghost fill
   return n;

@@ -181,7 +181,7 @@ __device__ __forceinline__ float recip(float x) {
   asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
   return r * fmaf(-x, r, 2.0f);
 }
-__device__ __forceinline__ double recip(double x) { return 1.0 / x; }
+MRTLB_HD double recip(double x) { return 1.0 / x; }
 // The same three functions on a pair of nodes (pair.cuh): the reciprocal's
 // Newton-Raphson step and the compensated numerator run packed; the
 // hardware approximation and the exponential run per lane.
@@ -256,8 +256,8 @@ MRTLB_HD R lw_update(const Coef<R>& c, int q, R f0, R Cq, R fE, R fW, R fN, R fS
   return v;
 }
 
-__device__ __forceinline__ float expr(float x) { return expf(x); }
-__device__ __forceinline__ double expr(double x) { return exp(x); }
+MRTLB_HD float expr(float x) { return expf(x); }
+MRTLB_HD double expr(double x) { return exp(x); }
 
 // Equilibrium moments k = 4..15 (Eqs. 14a-14i and the version rule for
 // k = 11, 14, 15), given the conserved moments and u, T.
