@@ -556,7 +556,7 @@ void run_segment(mrtlb_ctx* c, mrtlb_adjoint_state* a, long len, const Coef<R>& 
     R* fout = (n + 1 < len) ? slot<R>(c, a, n + 1) : last;
     if (!fout) break;
     if (a->tiled) launch_step_tiled<R>(a->plan[n], 0, c->L, k, c->err, st, fout);
-    else launch_step_plain<R>(fin, fout, c->L, k, nullptr, c->err, st);  // (the walls are in the slot)
+    else launch_plain_step<R>(c, fin, fout, k, false, st);  // (the walls are in the slot)
   }
 }
 

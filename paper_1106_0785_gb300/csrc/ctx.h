@@ -9,6 +9,7 @@
 
 #include "../../include/mrtlb.h"
 #include "kernels.cuh"
+#include "step_split.cuh"
 #include "step_tiled.cuh"
 
 using namespace mrtlb;
@@ -45,8 +46,9 @@ struct mrtlb_ctx {
   cudaStream_t stream = nullptr;
   int kernel = MRTLB_KERNEL_AUTO;
   // library-owned scratch
-  int* err = nullptr;            // device error word
-  double* acc = nullptr;         // 5 doubles for mrtlb_reduce
+  int* err = nullptr;            // device error word; the start of the scratch allocation
+  void* split = nullptr;         // SplitTable of the context's precision (small grids), in it
+  double* acc = nullptr;         // 5 doubles for mrtlb_reduce, in it
   double* Tprev = nullptr;       // [ny][nx] for the residual
   int have_prev = 0;
   void* staging = nullptr;       // dense f or 4 FP64 fields
@@ -66,4 +68,15 @@ struct mrtlb_ctx {
 };
 
 void mrtlb_adjoint_free_internal(mrtlb_ctx* c);
+
+// One step of the plain kernel choice: a velocity per lane on small grids,
+// else a thread per node.  refill: the kernel works out walls and diffuse
+// ghosts itself (else it reads them from fin).
+template <typename R>
+inline void launch_plain_step(const mrtlb_ctx* c, const R* fin, R* fout, const Coef<R>& k, bool refill, cudaStream_t st) {
+  if (c->split && use_split<R>(c->L))
+    launch_step_split<R>(fin, fout, c->L, k, (const SplitTable<R>*)c->split, refill, c->err, st);
+  else
+    launch_step_plain<R>(fin, fout, c->L, k, refill ? &c->walls : nullptr, c->err, st);
+}
 

@@ -37,6 +37,7 @@ __global__ void __launch_bounds__(128) step_plain_kernel(const R* __restrict__ f
   const long long P = L.plane;
   const long long at = L.node(i, j);
   const long long E = at + 1, W = at - 1, N = at + L.pitch, S = at - L.pitch;
+  after_previous();
 
   R f[16];
 #pragma unroll
@@ -88,19 +89,16 @@ void launch_step_plain(const R* fin, R* fout, const Layout& L, const Coef<R>& c,
   // a grid small enough to leave SMs idle takes blocks of fewer threads
   // (the smallest power of two, at least 8, that covers it with one block
   // per SM), so that its latency-bound nodes spread over every SM
-  static const int nsm = [] {  // thread-safe static initialisation
-    int dev = 0, n = 0;
-    cudaGetDevice(&dev);
-    if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n <= 0) n = 152;
-    return n;
-  }();
+  const int nsm = sm_count();
   const long long n = (long long)ni * nj;
   int blk = 8;
   while (blk < 128 && (long long)blk * nsm < n) blk *= 2;
   const unsigned grd = (unsigned)((n + blk - 1) / blk);
   const bool refill = w && wall_count(L) > 0;
-  if (refill) step_plain_kernel<R, true><<<grd, blk, 0, st>>>(fin, fout, L, c, *w, err);
-  else step_plain_kernel<R, false><<<grd, blk, 0, st>>>(fin, fout, L, c, Walls{}, err);
+  const auto kernel = refill ? step_plain_kernel<R, true> : step_plain_kernel<R, false>;
+  // (set up while the step before it runs: FP32 600 x 100 4.0 -> 3.7 us, 100 x 101
+  // 2.74 -> 2.26; FP64 gains nothing)
+  launch_chained(sizeof(R) == 4, kernel, grd, blk, st, fin, fout, L, c, refill ? *w : Walls{}, err);
 }
 
 // ---------------------------------------------------------------------------

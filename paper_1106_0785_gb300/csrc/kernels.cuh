@@ -214,6 +214,40 @@ __device__ __forceinline__ void wall_node(R* f, const Layout& L, const Coef<R>& 
   for (int q = 0; q < 16; ++q) f[q * P + at] = v[q];
 }
 
+// Consecutive small launches of one stream.  A kernel launched with `early`
+// may be set up (its blocks resident, its constants loaded) while the one
+// before it still runs; after_previous() holds it until that one has completed,
+// before it touches anything a kernel writes.  It lets its own successor start
+// after that point, not before: with several launches resident ahead of their
+// turn the blocks of one are placed unevenly (FP64, 1600 nodes: 5.5 -> 16.7 us
+// per step).
+__device__ __forceinline__ void after_previous() {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+template <typename... P, typename... A>
+inline void launch_chained(bool early, void (*kernel)(P...), unsigned grd, unsigned blk, cudaStream_t st, A... args) {
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = early ? 1 : 0;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(grd);
+  cfg.blockDim = dim3(blk);
+  cfg.stream = st;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  cudaLaunchKernelEx(&cfg, kernel, P(args)...);
+}
+inline int sm_count() {
+  static const int nsm = [] {  // thread-safe static initialisation
+    int dev = 0, n = 0;
+    cudaGetDevice(&dev);
+    if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n <= 0) n = 152;
+    return n;
+  }();
+  return nsm;
+}
+
 // One step by the one-thread-per-node kernel.  With `w` it works out the walls
 // and diffuse ghosts beside its nodes itself; without, it reads them from fin.
 template <typename R>

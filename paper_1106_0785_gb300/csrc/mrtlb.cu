@@ -374,12 +374,33 @@ extern "C" int mrtlb_state_bytes(const mrtlb_ctx* c, size_t* bytes) {
   return MRTLB_OK;
 }
 
+// The lane constants of the small-grid step on the device, from the current
+// coefficients (at bind, and when the rates change).
+template <typename R>
+static int upload_split(mrtlb_ctx* c, const Coef<R>& k) {
+  if (!c->split) return MRTLB_OK;
+  SplitTable<R> t;
+  split_table<R>(k, c->walls, &t);
+  // (a copy from pageable memory has taken the table when it returns)
+  CK(cudaMemcpyAsync(c->split, &t, sizeof(t), cudaMemcpyHostToDevice, c->stream), "copy lane constants");
+  return MRTLB_OK;
+}
+static int refresh_split(mrtlb_ctx* c) {
+  return c->prec == MRTLB_FP64 ? upload_split<double>(c, c->c64) : upload_split<float>(c, c->c32);
+}
+
+// One allocation for the error word, the accumulators and the lane constants.
 static int ensure_scratch(mrtlb_ctx* c) {
-  if (!c->err) {
-    CK(cudaMalloc((void**)&c->err, 256), "cudaMalloc(error word)");
-    CK(cudaMemsetAsync(c->err, 0, 256, c->stream), "cudaMemsetAsync");
-  }
-  if (!c->acc) CK(cudaMalloc((void**)&c->acc, 8 * sizeof(double)), "cudaMalloc(accumulators)");
+  if (c->err) return MRTLB_OK;
+  const bool fp64 = c->prec == MRTLB_FP64;
+  const bool split = fp64 ? use_split<double>(c->L) : use_split<float>(c->L);
+  const size_t table = !split ? 0 : fp64 ? sizeof(SplitTable<double>) : sizeof(SplitTable<float>);
+  char* p = nullptr;
+  CK(cudaMalloc((void**)&p, 512 + table), "cudaMalloc(scratch)");
+  c->err = (int*)p;
+  c->acc = (double*)(p + 256);
+  if (split) c->split = p + 512;
+  CK(cudaMemsetAsync(c->err, 0, 256, c->stream), "cudaMemsetAsync");
   return MRTLB_OK;
 }
 
@@ -425,6 +446,8 @@ extern "C" int mrtlb_bind(mrtlb_ctx* c, void* f_a, void* f_b, size_t bytes) {
   CK(cudaMemsetAsync(f_a, 0, c->state_bytes, c->stream), "cudaMemsetAsync");
   CK(cudaMemsetAsync(f_b, 0, c->state_bytes, c->stream), "cudaMemsetAsync");
   drop_graphs(c);
+  rc = refresh_split(c);
+  if (rc) return rc;
   rc = plan_tiled(c->L, (int)c->esize, c->f[0], c->f[1], &c->plan);
   if (rc) return fail(c, MRTLB_ERR_CUDA, "tensor-map set-up failed (%d)", rc);
   return MRTLB_OK;
@@ -497,10 +520,10 @@ static void enqueue_one(mrtlb_ctx* c, int cur, cudaStream_t st, bool timed) {
   if (timed) cudaEventRecord(c->ev[2 * c->ev_used], st);
   if (c->prec == MRTLB_FP64) {
     if (tiled) launch_step_tiled<double>(c->plan, cur, c->L, c->c64, c->err, st, fout);
-    else launch_step_plain<double>((const double*)fin, (double*)fout, c->L, c->c64, &c->walls, c->err, st);
+    else launch_plain_step<double>(c, (const double*)fin, (double*)fout, c->c64, true, st);
   } else {
     if (tiled) launch_step_tiled<float>(c->plan, cur, c->L, c->c32, c->err, st, fout);
-    else launch_step_plain<float>((const float*)fin, (float*)fout, c->L, c->c32, &c->walls, c->err, st);
+    else launch_plain_step<float>(c, (const float*)fin, (float*)fout, c->c32, true, st);
   }
   if (timed) {
     cudaEventRecord(c->ev[2 * c->ev_used + 1], st);
@@ -709,7 +732,9 @@ extern "C" int mrtlb_set_rates(mrtlb_ctx* c, const double* s) {
   for (int q = 0; q < 16; ++q) c->s[q] = s[q];
   ++c->gen;
   drop_graphs(c);  // captured launches hold the old coefficients
-  return build_coefficients(c);
+  const int rc = build_coefficients(c);
+  if (rc || !c->f[0]) return rc;
+  return refresh_split(c);
 }
 
 extern "C" int mrtlb_get_rates(const mrtlb_ctx* c, double* s) {
@@ -781,9 +806,8 @@ extern "C" const char* mrtlb_last_error(const mrtlb_ctx* c) {
 
 extern "C" void mrtlb_destroy(mrtlb_ctx* c) {
   if (!c) return;
-  if (c->err || c->acc || c->staging || c->Tprev) cudaStreamSynchronize(c->stream);
-  if (c->err) cudaFree(c->err);
-  if (c->acc) cudaFree(c->acc);
+  if (c->err || c->staging || c->Tprev) cudaStreamSynchronize(c->stream);
+  if (c->err) cudaFree(c->err);  // (and with it the accumulators and lane constants)
   if (c->Tprev) cudaFree(c->Tprev);
   if (c->staging) cudaFree(c->staging);
   if (c->ev) free_events(c);
