@@ -287,6 +287,9 @@ __global__ void init_eq_kernel(const double* __restrict__ rho_in, const double* 
 template <typename R>
 void launch_init_eq(const double* rho, const double* ux, const double* uy, const double* T, R* f,
                     const Layout& L, const Coef<double>& c64, cudaStream_t st) {
+  if constexpr (sizeof(R) == 4) {
+    if (launch_init_eq_df(rho, ux, uy, T, f, L, c64, st)) return;
+  }
   const long long n = (long long)L.ny * L.nx;
   init_eq_kernel<R><<<grid_for(n, 128), 128, 0, st>>>(rho, ux, uy, T, f, L, c64);
 }
@@ -325,11 +328,10 @@ void launch_macros(const R* f, double* rho, double* ux, double* uy, double* T, c
 }
 
 // ---------------------------------------------------------------------------
-// Conservation sums (FP64) and the max |T - T_prev| residual.
-// Warp shuffles, then one atomic per warp.
+// Conservation sums and the max |T - T_prev| residual of an FP64 state (of an
+// FP32 one: start.cu).  Warp shuffles, then one atomic per warp.
 // ---------------------------------------------------------------------------
-template <typename R>
-__global__ void reduce_kernel(const R* __restrict__ f, double* acc, double* Tprev, int have_prev,
+__global__ void reduce_kernel(const double* __restrict__ f, double* acc, double* Tprev, int have_prev,
                               Layout L) {
   const long long n = (long long)L.ny * L.nx;
   double s0 = 0, s1 = 0, s2 = 0, s3 = 0, mx = 0;
@@ -339,7 +341,7 @@ __global__ void reduce_kernel(const R* __restrict__ f, double* acc, double* Tpre
     const long long at = L.node(i, j);
     double g[16];
 #pragma unroll
-    for (int q = 0; q < 16; ++q) g[q] = (double)f[q * L.plane + at];
+    for (int q = 0; q < 16; ++q) g[q] = f[q * L.plane + at];
     double rho, jx, jy, e;
     conserved(g, rho, jx, jy, e);
     s0 += rho; s1 += jx; s2 += jy; s3 += e;
@@ -372,8 +374,12 @@ __global__ void reduce_kernel(const R* __restrict__ f, double* acc, double* Tpre
 template <typename R>
 void launch_reduce(const R* f, double* acc, double* Tprev, int have_prev, const Layout& L,
                    cudaStream_t st) {
-  const long long n = (long long)L.ny * L.nx;
-  reduce_kernel<R><<<grid_for(n, 256), 256, 0, st>>>(f, acc, Tprev, have_prev, L);
+  if constexpr (sizeof(R) == 4) {
+    launch_reduce_f32(f, acc, Tprev, have_prev, L, st);
+  } else {
+    const long long n = (long long)L.ny * L.nx;
+    reduce_kernel<<<grid_for(n, 256), 256, 0, st>>>(f, acc, Tprev, have_prev, L);
+  }
 }
 
 #define MRTLB_INSTANTIATE(R)                                                                     \

@@ -271,6 +271,11 @@ void launch_init_eq(const double* rho, const double* ux, const double* uy, const
 template <typename R>
 void launch_macros(const R* f, double* rho, double* ux, double* uy, double* T, const Layout& L,
                    cudaStream_t st);
+// FP32 states without the FP64 pipe (start.cu); the first is false for what it
+// does not do (version 3)
+bool launch_init_eq_df(const double* rho, const double* ux, const double* uy, const double* T, float* f, const Layout& L,
+                       const Coef<double>& c64, cudaStream_t st);
+void launch_reduce_f32(const float* f, double* acc, double* Tprev, int have_prev, const Layout& L, cudaStream_t st);
 // acc: 4 FP64 sums + 1 max (as the bit pattern of a non-negative double);
 // Tprev: [ny][nx] FP64 temperatures of the previous call (updated in place)
 template <typename R>
