@@ -159,7 +159,7 @@ __global__ void __launch_bounds__(128, sizeof(R) == 4 ? MRTLB_ADJ_MINB : 2)
     if (i <= L.nx && !((i < 0 || i >= L.nx) && (j < 0 || j >= L.ny)))
       adj_core_node<R, RATES>(ft, lam, Ux, Uy, gsh, gst, out, L, a, i, j, G);
   }
-  if constexpr (RATES) flush_rate_gradients(G, gacc);
+  if constexpr (RATES) flush_rate_gradients<R, 128>(G, gacc);
 }
 
 // Adjoint march shapes: 128-column strips (FP32; 64 for FP64, same box
@@ -572,7 +572,7 @@ int backward_impl(mrtlb_ctx* c, const double* dL_dmacros, const double* dL_dfK, 
   R* lam1 = (R*)a->lam[1];
   ACK(cudaMemsetAsync(lam0, 0, sb, st), "clear");
   ACK(cudaMemsetAsync(lam1, 0, sb, st), "clear");
-  ACK(cudaMemsetAsync(a->gacc, 0, 16 * sizeof(double), st), "clear");
+  ACK(cudaMemsetAsync(a->gacc, 0, kGradSlots * 16 * sizeof(double), st), "clear");
   // seed on B(f^K)
   R* fK = (R*)c->f[c->cur];
   launch_bc<R>(fK, L, k, c->walls, st);
@@ -609,7 +609,8 @@ int backward_impl(mrtlb_ctx* c, const double* dL_dmacros, const double* dL_dfK, 
     dim3 gd((L.nx + 127) / 128, L.ny, 16);
     adj_dense_kernel<R><<<gd, 128, 0, st>>>((R*)a->lam[li], dL_df0, L, 1);
   }
-  if (dL_ds) ACK(cudaMemcpyAsync(dL_ds, a->gacc, 16 * sizeof(double), cudaMemcpyDeviceToHost, st), "copy grads");
+  double grads[kGradSlots * 16];
+  if (dL_ds) ACK(cudaMemcpyAsync(grads, a->gacc, sizeof(grads), cudaMemcpyDeviceToHost, st), "copy grads");
   int h = 0;
   ACK(cudaMemcpyAsync(&h, c->err, sizeof(int), cudaMemcpyDeviceToHost, st), "read error word");
   ACK(cudaStreamSynchronize(st), "cudaStreamSynchronize");
@@ -617,7 +618,11 @@ int backward_impl(mrtlb_ctx* c, const double* dL_dmacros, const double* dL_dfK, 
   if (h & ERRBIT_NONPHYSICAL)  // (the gradients of such a run mean nothing)
     return afail(c, MRTLB_ERR_NONPHYSICAL, "a state of the forward pass was non-physical (rho <= 0, T <= 0 or not finite)");
   if (dL_ds)  // the kernels sum the rate gradients without the factor dt
-    for (int k = 0; k < 16; ++k) dL_ds[k] *= c->p.dt;
+    for (int k = 0; k < 16; ++k) {
+      double sum = 0.0;
+      for (int q = 0; q < kGradSlots; ++q) sum += grads[16 * q + k];
+      dL_ds[k] = sum * c->p.dt;
+    }
   return MRTLB_OK;
 }
 
@@ -646,7 +651,7 @@ int allocate(mrtlb_ctx* c, mrtlb_adjoint_state* a, long S, long nck) {
   ACK(cudaMalloc(&a->ux, pb), "cudaMalloc(u)");
   ACK(cudaMalloc(&a->uy, pb), "cudaMalloc(u)");
   for (void* q : {a->gsh, a->gst, a->ux, a->uy}) ACK(cudaMemsetAsync(q, 0, pb, st), "clear");
-  ACK(cudaMalloc((void**)&a->gacc, 16 * sizeof(double)), "cudaMalloc(grad)");
+  ACK(cudaMalloc((void**)&a->gacc, kGradSlots * 16 * sizeof(double)), "cudaMalloc(grad)");
   a->core_blocks = core_resident_blocks<R>();
   // one read map per slot for the tiled step (the write side is a plain pointer)
   TiledPlan p0;

@@ -338,15 +338,41 @@ __device__ __forceinline__ void velocity_T(R uxb, R uyb, R ux, R uy, R ir, R lt[
   for (int q = 0; q < 16; ++q) lt[q] += (uxb * (R(vx_of(q)) - ux) + uyb * (R(vy_of(q)) - uy)) * ir;
 }
 
-// Sum the rate gradients over the warp; one FP64 atomic per warp and rate.
-template <typename R>
+// Sum the rate gradients of a block of NT threads (all of them call it): over
+// each warp in R, then over its warps and into gacc in FP64, one atomic per
+// rate.  The 16 values of a warp's lanes are summed together: at each of four
+// stages a lane hands over half of the values it still holds, so the warp ends
+// with value k in lanes k and k + 16 after 16 shuffles and additions instead of
+// 60.  Blocks take turns at kGradSlots copies of the 12 sums, which the caller
+// adds up.  One atomic per warp and rate onto one copy had them queue: us per
+// adjoint step in FP32 on GB300 (two-pass kernels), 512 x 128 26.5 -> 18.2,
+// 200 x 100 19.4 -> 15.3, 700 x 500 54.4 -> 38.2.
+constexpr int kGradSlots = 32;
+template <typename R, int NT>
 __device__ __forceinline__ void flush_rate_gradients(const R G[16], double* gacc) {
+  __shared__ R part[NT / 32][16];
+  const int lane = threadIdx.x & 31;
+  R v[16];
 #pragma unroll
-  for (int k = 4; k < 16; ++k) {
-    R v = G[k];
+  for (int k = 0; k < 16; ++k) v[k] = (k < 4) ? R(0) : G[k];
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    if ((threadIdx.x & 31) == 0 && v != R(0)) atomicAdd(gacc + k, (double)v);
+  for (int o = 8; o > 0; o >>= 1) {  // keep the values whose index has the lane's bit o
+    const bool up = lane & o;
+#pragma unroll
+    for (int k = 0; k < o; ++k) {
+      const R give = up ? v[k] : v[k + o];
+      v[k] = (up ? v[k + o] : v[k]) + __shfl_xor_sync(0xffffffffu, give, o);
+    }
+  }
+  v[0] += __shfl_xor_sync(0xffffffffu, v[0], 16);
+  if (lane < 16) part[threadIdx.x >> 5][lane] = v[0];
+  __syncthreads();
+  if (threadIdx.x >= 4 && threadIdx.x < 16) {
+    double sum = 0.0;
+#pragma unroll
+    for (int w = 0; w < NT / 32; ++w) sum += (double)part[w][threadIdx.x];
+    const int slot = (int)((blockIdx.y * gridDim.x + blockIdx.x) % kGradSlots);
+    if (sum != 0.0) atomicAdd(gacc + 16 * slot + threadIdx.x, sum);
   }
 }
 

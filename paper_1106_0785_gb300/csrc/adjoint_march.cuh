@@ -278,7 +278,7 @@ __global__ void __launch_bounds__(BX, sizeof(R) == 4 ? 3 : 1)
     if (m.t == 0) atomicOr(err, ERRBIT_TIMEOUT);
     m.drain();
   }
-  if constexpr (RATES) flush_rate_gradients(G, gacc);
+  if constexpr (RATES) flush_rate_gradients<R, BX>(G, gacc);
 }
 
 }  // namespace
