@@ -82,7 +82,7 @@ __device__ __forceinline__ R gbar_at(const R* gb, const Layout& L, int i, int j)
 
 // Pass 2: lambda~(p) for one node p of [-1, nx] x [-1, ny] (corners
 // excluded); the rate gradients of an advanced node are added to G.
-template <typename R, bool RATES>
+template <typename R, bool RATES, int VER>
 __device__ __forceinline__ void adj_core_node(const R* __restrict__ ft, const R* __restrict__ lam,
                                               const R* __restrict__ Ux, const R* __restrict__ Uy,
                                               const R* __restrict__ gsh, const R* __restrict__ gst,
@@ -116,7 +116,7 @@ __device__ __forceinline__ void adj_core_node(const R* __restrict__ ft, const R*
     const long long aE = at + 1, aW = at - 1, aN = at + L.pitch, aS = at - L.pitch;
     const R shear = (Ux[aE] - Ux[aW]) * c.inv2dx - (Uy[aN] - Uy[aS]) * c.inv2dy;
     const R strain = (Uy[aE] - Uy[aW]) * c.inv2dx + (Ux[aN] - Ux[aS]) * c.inv2dy;
-    collision_T_node<R, RATES>(a, g, lp, ux, uy, shear, strain, uxb, uyb, lt, G);
+    collision_T_node<R, RATES, VER>(a, g, lp, ux, uy, shear, strain, uxb, uyb, lt, G);
   } else if (c.modified) {
     velocity_T(uxb, uyb, ux, uy, ir, lt);
   }
@@ -145,7 +145,7 @@ __device__ __forceinline__ void adj_core_node(const R* __restrict__ ft, const R*
 // Persistent over row tiles of 128 nodes (tile t: row -1 + t / tiles_x);
 // each thread sums the rate gradients of all its nodes before the warp
 // reduction.
-template <typename R, bool RATES>
+template <typename R, bool RATES, int VER>
 __global__ void __launch_bounds__(128, sizeof(R) == 4 ? MRTLB_ADJ_MINB : 2)
     adj_core_kernel(const R* __restrict__ ft, const R* __restrict__ lam, const R* __restrict__ Ux,
                     const R* __restrict__ Uy, const R* __restrict__ gsh, const R* __restrict__ gst,
@@ -157,7 +157,7 @@ __global__ void __launch_bounds__(128, sizeof(R) == 4 ? MRTLB_ADJ_MINB : 2)
     const int i = -1 + (t % tiles_x) * 128 + (int)threadIdx.x;
     const int j = -1 + t / tiles_x;
     if (i <= L.nx && !((i < 0 || i >= L.nx) && (j < 0 || j >= L.ny)))
-      adj_core_node<R, RATES>(ft, lam, Ux, Uy, gsh, gst, out, L, a, i, j, G);
+      adj_core_node<R, RATES, VER>(ft, lam, Ux, Uy, gsh, gst, out, L, a, i, j, G);
   }
   if constexpr (RATES) flush_rate_gradients<R, 128>(G, gacc);
 }
@@ -247,13 +247,19 @@ __global__ void adj_diffuse_kernel(R* lam, Layout L, Coef<R> c, Walls w, int sid
   }
 }
 
-// B^T, walls on one side: the wall node w was NEE(f(a)) of its fluid
-// neighbour a: lambda(a) += (dNEE/df(a))^T lambda~(w), lambda(w) = 0.
+// B^T, walls: the wall node w was NEE(f(a)) of its fluid neighbour a:
+// lambda(a) += (dNEE/df(a))^T lambda~(w), lambda(w) = 0.  Threads 0 .. n-1 take
+// side `side`, the next n (if any) side + 1.
 template <typename R>
-__global__ void adj_walls_kernel(R* lam, const R* __restrict__ ft, Layout L, Coef<double> c, Walls w, int side) {
-  const int k = blockIdx.x * blockDim.x + threadIdx.x;
+__global__ void __launch_bounds__(32) adj_walls_kernel(R* lam, const R* __restrict__ ft, Layout L, Coef<double> c, Walls w,
+                                                       int side, int total) {
+  int k = blockIdx.x * blockDim.x + threadIdx.x;
+  if (k >= total) return;
   const int n = (side < 2) ? L.ny : L.nx;
-  if (k >= n) return;
+  if (k >= n) {
+    k -= n;
+    ++side;
+  }
   int i, j, ia, ja;
   if (side == 0) { i = 0; j = k; ia = 1; ja = k; }
   else if (side == 1) { i = L.nx - 1; j = k; ia = L.nx - 2; ja = k; }
@@ -271,18 +277,14 @@ __global__ void adj_walls_kernel(R* lam, const R* __restrict__ ft, Layout L, Coe
   const double ir = 1.0 / rho;
   const double ux = jx * ir, uy = jy * ir;
   const double T = temperature(rho, jx, jy, e, ir);
-  // NEE(g) = g + M^-1 (eq(rho, rho u_w, e_w, u_w, T_w) - eq(rho, j, e, u, T))
-  double db[16];
-  inverse_T(c, v, db, true);
-  const double uwx = w.ux[side], uwy = w.uy[side], Tw = w.T[side];
-  const double kw = Tw + 0.5 * (uwx * uwx + uwy * uwy);
-  EqIn<double> xw{rho, ir, rho * uwx, rho * uwy, rho * kw, uwx, uwy, Tw};
-  EqIn<double> gw{0, 0, 0, 0, 0, 0, 0, 0};
-  equilibrium_T(c, xw, db, gw);
-  double rbw = gw.rho - gw.ir * ir * ir + gw.jx * uwx + gw.jy * uwy + gw.e * kw;
-  double ndb[16];
+  // NEE(g) = g + rho f^eq(1, u_w, T_w) - M^-1 eq(rho, j, e, u, T)
+  double rbw = 0.0;
 #pragma unroll
-  for (int q = 0; q < 16; ++q) ndb[q] = -db[q];
+  for (int q = 0; q < 16; ++q) rbw += v[q] * w.e64[side][q];
+  double ndb[16];
+  inverse_T(c, v, ndb, true);
+#pragma unroll
+  for (int q = 0; q < 16; ++q) ndb[q] = -ndb[q];
   EqIn<double> xa{rho, ir, jx, jy, e, ux, uy, T};
   EqIn<double> ga{0, 0, 0, 0, 0, 0, 0, 0};
   equilibrium_T(c, xa, ndb, ga);
@@ -295,6 +297,19 @@ __global__ void adj_walls_kernel(R* lam, const R* __restrict__ ft, Layout L, Coe
     const double add = v[q] + rb + jxb * vx + jyb * vy + eb * 0.5 * (vx * vx + vy * vy);
     lam[q * P + aa] = (R)((double)lam[q * P + aa] + add);
     lam[q * P + aw] = R(0);
+  }
+}
+
+// Both walls of an axis in one launch, unless they share their fluid nodes.
+template <typename R>
+void launch_adj_walls(R* lam, const R* ft, const Layout& L, const Coef<double>& c, const Walls& w, cudaStream_t st) {
+  for (int s = 0; s < 4; ++s) {
+    if (L.bc[s] != BC_WALL) continue;
+    const int n = (s < 2) ? L.ny : L.nx, across = (s < 2) ? L.nx : L.ny;
+    const bool both = (s & 1) == 0 && L.bc[s + 1] == BC_WALL && across > 3;
+    const int total = both ? 2 * n : n;
+    adj_walls_kernel<R><<<(total + 31) / 32, 32, 0, st>>>(lam, ft, L, c, w, s, total);
+    if (both) ++s;
   }
 }
 
@@ -404,7 +419,7 @@ int core_resident_blocks() {
   int dev = 0, nsm = 1, per = 1;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, adj_core_kernel<R, true>, 128, 0);
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, adj_core_kernel<R, true, 0>, 128, 0);
   return std::max(1, nsm) * std::max(1, per);
 #endif
 }
@@ -482,21 +497,19 @@ void adjoint_step(mrtlb_ctx* c, mrtlb_adjoint_state* a, long n, int li, const Co
     adj_prep_kernel<R><<<g2, 128, 0, st>>>(ft, lam_in, (R*)a->ux, (R*)a->uy, (R*)a->gsh, (R*)a->gst, L, ac);
     const int ntiles = (int)(g2.x * g2.y);
     const int grid = std::min(ntiles, a->core_blocks);
-    if (rates)
-      adj_core_kernel<R, true><<<grid, 128, 0, st>>>(ft, lam_in, (const R*)a->ux, (const R*)a->uy, (const R*)a->gsh,
-                                                     (const R*)a->gst, lam_out, L, ac, a->gacc, (int)g2.x, ntiles);
-    else
-      adj_core_kernel<R, false><<<grid, 128, 0, st>>>(ft, lam_in, (const R*)a->ux, (const R*)a->uy, (const R*)a->gsh,
-                                                      (const R*)a->gst, lam_out, L, ac, a->gacc, (int)g2.x, ntiles);
+    const bool v1 = ac.c.version == 1;  // (as the march: version 1 without the others' transposes)
+    const auto core = rates ? (v1 ? adj_core_kernel<R, true, 1> : adj_core_kernel<R, true, 0>)
+                            : (v1 ? adj_core_kernel<R, false, 1> : adj_core_kernel<R, false, 0>);
+    core<<<grid, 128, 0, st>>>(ft, lam_in, (const R*)a->ux, (const R*)a->uy, (const R*)a->gsh, (const R*)a->gst, lam_out,
+                               L, ac, a->gacc, (int)g2.x, ntiles);
   }
   const int perim = 2 * L.nx + 2 * L.ny;
   adj_ghosts_kernel<R><<<dim3((perim + 127) / 128, 16), 128, 0, st>>>(lam_out, L);
   for (int s = 0; s < 4; ++s) {
     const int nn = (s < 2) ? L.ny : L.nx;
     if (L.bc[s] == BC_DIFFUSE) adj_diffuse_kernel<R><<<(nn + 127) / 128, 128, 0, st>>>(lam_out, L, k, c->walls, s);
-    if (L.bc[s] == BC_WALL)
-      adj_walls_kernel<R><<<(nn + 127) / 128, 128, 0, st>>>(lam_out, ft, L, c->c64, c->walls, s);
   }
+  launch_adj_walls<R>(lam_out, ft, L, c->c64, c->walls, st);
 }
 
 // Maps and row segments of the adjoint march; false if it cannot run.
@@ -583,11 +596,7 @@ int backward_impl(mrtlb_ctx* c, const double* dL_dmacros, const double* dL_dfK, 
     adj_dense_kernel<R><<<gd, 128, 0, st>>>(lam0, (double*)dL_dfK, L, dL_dmacros ? 2 : 0);
   }
   // walls of B^T for the seed
-  for (int s = 0; s < 4; ++s)
-    if (L.bc[s] == BC_WALL) {
-      const int n = (s < 2) ? L.ny : L.nx;
-      adj_walls_kernel<R><<<(n + 127) / 128, 128, 0, st>>>(lam0, fK, L, c->c64, c->walls, s);
-    }
+  launch_adj_walls<R>(lam0, fK, L, c->c64, c->walls, st);
   ACK(cudaGetLastError(), "adjoint seed");
   int li = 0;  // lambda[li] holds dL/df of the latest state reached
   const long K = a->K, S = a->S;
