@@ -676,7 +676,13 @@ int allocate(mrtlb_ctx* c, mrtlb_adjoint_state* a, long S, long nck) {
       }
     }
   }
-  a->march = a->tiled && plan_adj_march<R>(c, a);
+  // the fused march of the adjoint step, or the two-pass kernels: us per step on
+  // GB300, two-pass / march, FP32 512 x 128 18.2 / 21.5, 1024 x 256 31.5 / 25.6;
+  // FP64, bound by its instructions, of which the march has as many and more
+  // halo, 700 x 500 463 / 503
+  const long long nodes = (long long)c->L.nx * c->L.ny;
+  const bool march = c->kernel == MRTLB_KERNEL_AUTO ? nodes >= (fp64 ? 450000 : 130000) : c->kernel == MRTLB_KERNEL_TILED;
+  a->march = march && plan_adj_march<R>(c, a);
   return MRTLB_OK;
 }
 

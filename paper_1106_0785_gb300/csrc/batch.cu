@@ -26,7 +26,7 @@
 #include <vector>
 
 #include "ctx.h"
-#include "march.cuh"
+#include "march_f64.cuh"
 #include "march_pair.cuh"
 
 namespace mrtlb {
@@ -49,43 +49,35 @@ struct WallInst {
   int first;  // index of this instance's first wall node in the flat enumeration
 };
 
-template <typename R, int BX, int NSLOT>
-__host__ __device__ constexpr size_t batch_coef_off() {
-  return (Smem<R, BX, NSLOT>::bytes + 127) & ~(size_t)127;
-}
-template <typename R, int BX, int NSLOT>
-__host__ __device__ constexpr size_t batch_smem() {
-  return batch_coef_off<R, BX, NSLOT>() + sizeof(Coef<R>);
-}
+constexpr size_t kBatch64Coef = (March64::SM::bytes + 127) & ~(size_t)127;
+constexpr size_t kBatch64Smem = kBatch64Coef + sizeof(Coef<double>);
 
-template <typename R, int BX, int NSLOT, int MINB>
-__global__ void __launch_bounds__(BX, MINB) step_batched_kernel(const BatchInst<R>* __restrict__ insts,
-                                                                const int4* __restrict__ tiles, int ntiles,
-                                                                int cur, int* err) {
-  using SM = Smem<R, BX, NSLOT>;
+__global__ void __launch_bounds__(kRow64) step_batched_f64_kernel(const BatchInst<double>* __restrict__ insts,
+                                                                  const int4* __restrict__ tiles, int ntiles,
+                                                                  int cur, int* err) {
+  using SM = March64::SM;
   extern __shared__ __align__(128) unsigned char smem_raw[];
-  Coef<R>* cs = reinterpret_cast<Coef<R>*>(smem_raw + batch_coef_off<R, BX, NSLOT>());
-  March<R, BX, NSLOT> m;
-  m.slots = reinterpret_cast<R*>(smem_raw);
-  m.U = reinterpret_cast<R*>(smem_raw + SM::u_off);
+  Coef<double>* cs = reinterpret_cast<Coef<double>*>(smem_raw + kBatch64Coef);
+  March64 m;
+  m.slots = reinterpret_cast<double*>(smem_raw);
+  m.U = reinterpret_cast<double*>(smem_raw + SM::u_off);
   m.bars = reinterpret_cast<uint64_t*>(smem_raw + SM::bar_off);
   m.err = err;
   m.t = threadIdx.x;
   m.kbase = 0;
   if (m.t == 0) {
-    for (int s = 0; s < NSLOT; ++s) mbar_init(&m.bars[s], 1);
+    for (int s = 0; s < kSlot64; ++s) mbar_init(&m.bars[s], 1);
     mbar_fence_init();
   }
   for (int ti = blockIdx.x; ti < ntiles; ti += gridDim.x) {
     const int4 tl = tiles[ti];  // (instance, x0, ja, jb)
-    const BatchInst<R>* in = insts + tl.x;
+    const BatchInst<double>* in = insts + tl.x;
     {
       const uint32_t* src = reinterpret_cast<const uint32_t*>(&in->c);
       uint32_t* dst = reinterpret_cast<uint32_t*>(cs);
-      for (int k = m.t; k < (int)(sizeof(Coef<R>) / 4); k += BX) dst[k] = src[k];
+      for (int k = m.t; k < (int)(sizeof(Coef<double>) / 4); k += kRow64) dst[k] = src[k];
     }
     m.L = in->L;
-    m.plane = m.L.plane;
     m.map = &in->map[cur];
     m.fout = in->f[cur ^ 1];
     __syncthreads();  // coefficients in place (and the previous tile done with them)
@@ -192,43 +184,28 @@ __global__ void walls_batched_kernel(const WallInst* __restrict__ wi, int nw, in
   wall_node<R>(reinterpret_cast<R*>(w.f[cur]), w.L, c, w.w, g - w.first);
 }
 
-// kernel variants by strip width
-template <typename R> struct BatchShapes;
-template <> struct BatchShapes<float> {
-  static constexpr int NS = 4;
-};
-template <> struct BatchShapes<double> {
-  static constexpr int NS = 4;
-};
-
-#ifndef MRTLB_PAIR
-#define MRTLB_PAIR 1
-#endif
+constexpr int kBatchSlots = 4;  // rows in flight of the FP32 kernel
 
 // The dynamic shared memory the batched kernel of this shape needs, allowed
 // for it in the current context (set by set_tiles, so once per batch and
 // tile shape, on the batch's device, outside any stream capture).
 template <typename R, int BX, int MINB>
 cudaError_t allow_batched_smem() {
-  constexpr int NS = BatchShapes<R>::NS;
   const auto A = cudaFuncAttributeMaxDynamicSharedMemorySize;
-  if constexpr (sizeof(R) == 4 && MRTLB_PAIR)
-    return cudaFuncSetAttribute(step_batched_pair_kernel<BX, NS, MINB>, A, (int)batch_pair_smem<BX, NS>());
+  if constexpr (sizeof(R) == 4)
+    return cudaFuncSetAttribute(step_batched_pair_kernel<BX, kBatchSlots, MINB>, A, (int)batch_pair_smem<BX, kBatchSlots>());
   else
-    return cudaFuncSetAttribute(step_batched_kernel<R, BX, NS, MINB>, A, (int)batch_smem<R, BX, NS>());
+    return cudaFuncSetAttribute(step_batched_f64_kernel, A, (int)kBatch64Smem);
 }
 
 template <typename R, int BX, int MINB>
 void launch_batched_bx(const void* insts, const int4* tiles, int ntiles, int grid, int cur, int* err, int* claim,
                        cudaStream_t st) {
-  constexpr int NS = BatchShapes<R>::NS;
-  if constexpr (sizeof(R) == 4 && MRTLB_PAIR) {
-    step_batched_pair_kernel<BX, NS, MINB><<<grid, BX / 2, batch_pair_smem<BX, NS>(), st>>>(
+  if constexpr (sizeof(R) == 4)
+    step_batched_pair_kernel<BX, kBatchSlots, MINB><<<grid, BX / 2, batch_pair_smem<BX, kBatchSlots>(), st>>>(
         (const BatchInst<float>*)insts, tiles, ntiles, cur, err, claim);
-  } else {
-    step_batched_kernel<R, BX, NS, MINB><<<grid, BX, batch_smem<R, BX, NS>(), st>>>(
-        (const BatchInst<R>*)insts, tiles, ntiles, cur, err);
-  }
+  else
+    step_batched_f64_kernel<<<grid, kRow64, kBatch64Smem, st>>>((const BatchInst<double>*)insts, tiles, ntiles, cur, err);
 }
 
 }  // namespace

@@ -204,6 +204,20 @@ static int build_coefficients(mrtlb_ctx* c) {
       if (std::fabs(back[r] - (r == q ? 1.0 : 0.0)) > 1e-14)
         return fail(c, MRTLB_ERR_SINGULAR, "factorised inverse of M failed its check");
   }
+  for (int s = 0; s < 4; ++s) {
+    k.fS[s][0] = k.invS[s][2] * k.rate[10];
+    k.fS[s][1] = k.invS[s][3] * k.rate[11];
+    k.fX[s][0] = k.invX[s][2] * k.rate[8];
+    k.fX[s][1] = k.invX[s][3] * k.rate[14];
+    k.fY[s][0] = k.invY[s][2] * k.rate[9];
+    k.fY[s][1] = k.invY[s][3] * k.rate[15];
+  }
+  for (int s = 0; s < 2; ++s) {
+    k.fQ[s][0] = k.invQ[s][0] * k.rate[4];
+    k.fQ[s][1] = k.invQ[s][1] * k.rate[12];
+    k.fP[s][0] = k.invP[s][0] * k.rate[5];
+    k.fP[s][1] = k.invP[s][1] * k.rate[13] * 2.0;
+  }
   // FP32 copy
   Coef<float>& f = c->c32;
   f.a1x = (float)k.a1x; f.b1x = (float)k.b1x; f.a1y = (float)k.a1y; f.b1y = (float)k.b1y;

@@ -38,8 +38,16 @@ __host__ __device__ constexpr int vy_of(int q) {
 // Per-context constants.  The family inverse columns are pre-scaled by the
 // inverse-butterfly factors (1/4 for S and Q and 1/2 for X and Y on axis
 // shells, 1/4 for everything on diagonal shells).
+// FP64 only (the FP64 march): the columns of M^-1 that meet m - m^eq, times the
+// rates: moments 10, 11 (S), 8, 14 (X), 9, 15 (Y), 4, 12 (Q), 5, 13 / 2 (P).
 template <typename R>
-struct Coef {
+struct CoefFold {};
+template <>
+struct CoefFold<double> {
+  double fS[4][2], fX[4][2], fY[4][2], fQ[2][2], fP[2][2];
+};
+template <typename R>
+struct Coef : CoefFold<R> {
   // Lax-Wendroff (Sec. III): for unit speed along x, a1x = dt/(2dx),
   // b1x = (dt/dx)^2/2; speed-2 velocities use 2*a1x and 4*b1x.
   R a1x, b1x, a1y, b1y;

@@ -3,9 +3,10 @@
 // side of the march lives in march.cuh.
 #include <cuda.h>
 
+#include <algorithm>
 #include <cstddef>
 
-#include "march.cuh"
+#include "march_f64.cuh"
 #include "march_pair.cuh"
 #include "step_tiled.cuh"
 
@@ -13,34 +14,33 @@ namespace mrtlb {
 
 namespace {
 
-template <typename R, int BX, int NSLOT, int MINB>
-__global__ void __launch_bounds__(BX, MINB) step_tiled_kernel(const __grid_constant__ CUtensorMap tmap,
-                                                              R* __restrict__ fout, const Layout L,
-                                                              const Coef<R> c, int* err, const int seglen) {
-  using SM = Smem<R, BX, NSLOT>;
+__global__ void __launch_bounds__(kRow64) step_f64_kernel(const __grid_constant__ CUtensorMap tmap,
+                                                          double* __restrict__ fout, const Layout L,
+                                                          const __grid_constant__ Coef<double> c, int* err,
+                                                          const int seglen) {
+  using SM = March64::SM;
   extern __shared__ __align__(128) unsigned char smem_raw[];
   const int ja = L.j0 + blockIdx.y * seglen;
   const int jb = min(ja + seglen, L.j1);
   if (ja >= jb) return;  // uniform over the CTA
-  March<R, BX, NSLOT> m;
-  m.slots = reinterpret_cast<R*>(smem_raw);
-  m.U = reinterpret_cast<R*>(smem_raw + SM::u_off);
+  March64 m;
+  m.slots = reinterpret_cast<double*>(smem_raw);
+  m.U = reinterpret_cast<double*>(smem_raw + SM::u_off);
   m.bars = reinterpret_cast<uint64_t*>(smem_raw + SM::bar_off);
   m.map = &tmap;
   m.fout = fout;
   m.err = err;
-  m.plane = L.plane;
   m.L = L;
   m.t = threadIdx.x;
   m.kbase = 0;
   if (m.t == 0) {
-    for (int s = 0; s < NSLOT; ++s) mbar_init(&m.bars[s], 1);
+    for (int s = 0; s < kSlot64; ++s) mbar_init(&m.bars[s], 1);
     mbar_fence_init();
   }
   __syncthreads();
   // strips start on multiples of BX so that every TMA box starts on a
   // 16-byte boundary (xoff - HL and BX are multiples of 16 bytes)
-  if (m.segment(c, blockIdx.x * BX, ja, jb)) {
+  if (m.segment(c, blockIdx.x * kRow64, ja, jb)) {
     if (m.t == 0) atomicOr(err, ERRBIT_TIMEOUT);
     m.drain();
   }
@@ -51,16 +51,8 @@ __global__ void __launch_bounds__(BX, MINB) step_tiled_kernel(const __grid_const
 // bound of five CTAs (168 registers: three warps share an SM sub-partition's
 // register file) was 7% slower, 64-column strips with eight one-warp CTAs
 // 5% slower.
-#ifndef MRTLB_PAIR_MAXNREG
-#define MRTLB_PAIR_MAXNREG 0
-#endif
 template <int BX, int NSLOT, int MINB>
-__global__ void
-#if MRTLB_PAIR_MAXNREG > 0
-    __maxnreg__(MRTLB_PAIR_MAXNREG)
-#else
-    __launch_bounds__(BX / 2, MINB)
-#endif
+__global__ void __launch_bounds__(BX / 2, MINB)
     step_pair_kernel(const __grid_constant__ CUtensorMap tmap, float* __restrict__ fout, const Layout L,
                      const __grid_constant__ Coef<P2> c, int* err, const int seglen) {
   using SM = PairSmem<BX, NSLOT>;
@@ -120,21 +112,8 @@ EncodeFn get_encode() {
   return fn;
 }
 
-// tile shapes: FP32 128-node strips, 4-slot ring, 4 CTAs per SM;
-// FP64 64-node strips (same box bytes), 4-slot ring
-template <typename R> struct Tile;
-#ifndef MRTLB_PAIR_BX
-#define MRTLB_PAIR_BX 128
-#endif
-template <> struct Tile<float> { static constexpr int BX = MRTLB_PAIR_BX, NSLOT = 4, MINB = 4; };
-template <> struct Tile<double> { static constexpr int BX = 64, NSLOT = 4, MINB = 1; };
-
-#ifndef MRTLB_PAIR
-#define MRTLB_PAIR 1
-#endif
-#ifndef MRTLB_PAIR_MINB
-#define MRTLB_PAIR_MINB 4
-#endif
+// FP32 strips and ring
+constexpr int kPairBX = 128, kPairSlots = 4, kPairBlocks = 4;
 
 // The FP32 coefficient block with every constant in both lanes of a pair.
 Coef<P2> pair_coef(const Coef<float>& c) {
@@ -165,6 +144,30 @@ void plan_segments(const Layout& L, int target_ctas, TiledPlan* plan) {
   plan->nseg = (nj + seglen - 1) / seglen;
 }
 
+// FP64: segments of the length with the least FP64 instructions on the busiest
+// SM sub-partition (its warps take turns): a segment costs its rows and the two
+// arrivals around them, and a pair of CTAs has a warp on each sub-partition.
+// Returns whether that is less than the plain kernels take: the march's 275 a
+// row and lane against 508 a node with 32 nodes a warp, or 60 with two.
+static bool plan_f64(const Layout& L, int nsm, TiledPlan* plan) {
+  const int nj = std::max(1, L.j1 - L.j0);
+  const long long n = (long long)(L.i1 - L.i0) * nj;
+  long long best = -1;
+  for (int len = 1; len <= std::min(nj, 512); ++len) {
+    const long long ctas = (long long)plan->nstrips * ((nj + len - 1) / len);
+    const long long turns = ((ctas + nsm - 1) / nsm + 1) / 2;
+    const long long cost = turns * (275LL * len + 110) + 40;  // (40: the first rows' latency)
+    if (best < 0 || cost <= best) {
+      best = cost;
+      plan->seglen = len;
+    }
+  }
+  plan->nseg = (nj + plan->seglen - 1) / plan->seglen;
+  const long long lanes = 128LL * nsm;  // 32 lanes on each of 4 sub-partitions
+  const long long plain = 508 * ((n + lanes - 1) / lanes), split = 60 * ((16 * n + lanes - 1) / lanes);
+  return best < plain && best < split;
+}
+
 int plan_tiled(const Layout& L, int esize, void* f0, void* f1, TiledPlan* plan) {
   plan->ok = false;
   plan->esize = esize;
@@ -174,50 +177,22 @@ int plan_tiled(const Layout& L, int esize, void* f0, void* f1, TiledPlan* plan) 
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
   if (nsm <= 0) nsm = 152;
-  int minb;
-  if (esize == 4) {
-    plan->bx = Tile<float>::BX;
-    plan->nslot = Tile<float>::NSLOT;
-    plan->smem = Smem<float, Tile<float>::BX, Tile<float>::NSLOT>::bytes;
-    minb = Tile<float>::MINB;
-  } else {
-    plan->bx = Tile<double>::BX;
-    plan->nslot = Tile<double>::NSLOT;
-    plan->smem = Smem<double, Tile<double>::BX, Tile<double>::NSLOT>::bytes;
-    minb = 3;
-  }
+  plan->bx = (esize == 4) ? kPairBX : kRow64;
   const int rc = encode_row_maps(L, esize, f0, f1, plan->bx, plan->map);
   if (rc) return rc;
-  // resident CTAs per SM (shared memory and the launch bound); one full wave
-  int per_sm = (int)((227 * 1024) / (plan->smem + 1024));
-  if (per_sm > minb) per_sm = minb;
-  if (esize == 4 && MRTLB_PAIR) {  // the kernel launched for FP32: ask the runtime
-    constexpr int BX = Tile<float>::BX, NS = Tile<float>::NSLOT;
-    int n = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, step_pair_kernel<BX, NS, MRTLB_PAIR_MINB>, BX / 2,
-                                                      PairSmem<BX, NS>::bytes) == cudaSuccess && n > 0)
-      per_sm = n;
-    plan->smem = PairSmem<BX, NS>::bytes;
-  }
-  if (per_sm < 1) per_sm = 1;
   // the dynamic shared memory of the kernel launch_step_tiled will launch,
   // allowed in the current context (here: once per bind, on the bound
-  // device, outside any stream capture)
-  {
-    const auto A = cudaFuncAttributeMaxDynamicSharedMemorySize;
-    constexpr int BXf = Tile<float>::BX, NSf = Tile<float>::NSLOT, MBf = Tile<float>::MINB;
-    constexpr int BXd = Tile<double>::BX, NSd = Tile<double>::NSLOT, MBd = Tile<double>::MINB;
-    cudaError_t e;
-    if (esize == 4 && MRTLB_PAIR)
-      e = cudaFuncSetAttribute(step_pair_kernel<BXf, NSf, MRTLB_PAIR_MINB>, A, (int)PairSmem<BXf, NSf>::bytes);
-    else if (esize == 4)
-      e = cudaFuncSetAttribute(step_tiled_kernel<float, BXf, NSf, MBf>, A, (int)Smem<float, BXf, NSf>::bytes);
-    else
-      e = cudaFuncSetAttribute(step_tiled_kernel<double, BXd, NSd, MBd>, A, (int)Smem<double, BXd, NSd>::bytes);
-    if (e != cudaSuccess) {
-      cudaGetLastError();
-      return 4;
-    }
+  // device, outside any stream capture), and its resident CTAs per SM
+  const auto pair = step_pair_kernel<kPairBX, kPairSlots, kPairBlocks>;
+  plan->smem = (esize == 4) ? PairSmem<kPairBX, kPairSlots>::bytes : March64::SM::bytes;
+  const void* kernel = (esize == 4) ? (const void*)pair : (const void*)step_f64_kernel;
+  int per_sm = 0;
+  if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)plan->smem) != cudaSuccess ||
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, esize == 4 ? kPairBX / 2 : kRow64, plan->smem) !=
+          cudaSuccess ||
+      per_sm < 1) {
+    cudaGetLastError();
+    return 4;
   }
   // One wave of resident CTAs; for the FP32 march the most waves, up to
   // four, whose segments keep at least kWaveRows rows (each wave then marches
@@ -230,7 +205,7 @@ int plan_tiled(const Layout& L, int esize, void* f0, void* f1, TiledPlan* plan) 
   // last strip); a partial last wave (1.5 waves: 0.118 on 4096 x 1024)
   // leaves SMs idle.
   plan_segments(L, nsm * per_sm, plan);
-  if (esize == 4 && MRTLB_PAIR) {
+  if (esize == 4) {
     constexpr int kWaveRows = 24;
     for (int waves = 4; waves >= 2; --waves) {
       TiledPlan more = *plan;
@@ -243,13 +218,12 @@ int plan_tiled(const Layout& L, int esize, void* f0, void* f1, TiledPlan* plan) 
       }
     }
   }
-  // The CTAs with which a march of short segments (8 rows or more) beats the
-  // plain kernel, measured on GB300, us per step, plain / march: FP32 700 x 500
+  // FP32: the CTAs with which a march of short segments (8 rows or more) beats
+  // the plain kernel, measured on GB300, us per step, plain / march: 700 x 500
   // (2.5 CTAs per SM) 13.4 / 16.7, 1501 x 300 (3.0) 16.5 / 15.4, 1000 x 600
-  // (3.9) 23.1 / 16.1, 1501 x 701 (segments of 15 rows) 44.1 / 28.4; FP64
-  // 1024 x 128 (1.7) 132 / 130, 1000 x 150 (2.0) 151 / 130, 1024 x 256 (3.0)
-  // 262 / 225.
-  plan->fill = (esize == 4 ? 3 : 2) * nsm;
+  // (3.9) 23.1 / 16.1, 1501 x 701 (segments of 15 rows) 44.1 / 28.4.
+  if (esize == 4) plan->pays = plan->seglen >= kMinMarchRows || plan->nstrips * plan->nseg >= 3 * nsm;
+  else plan->pays = plan_f64(L, nsm, plan);
   plan->ok = true;
   return 0;
 }
@@ -281,27 +255,19 @@ bool use_tiled(int which, const TiledPlan& plan, bool fp64) {
   if (!plan.ok) return false;
   if (which == MRTLB_KERNEL_PLAIN) return false;
   if (which == MRTLB_KERNEL_TILED) return true;
-  // AUTO: a march of a few rows is latency-bound (each row waits for its
-  // copy) unless there are enough of them to fill the device; smaller grids
-  // go to the one-thread-per-node kernel
-  return plan.seglen >= kMinMarchRows || plan.nstrips * plan.nseg >= plan.fill;
+  return plan.pays;
 }
 
 template <typename R>
 void launch_step_tiled(const TiledPlan& plan, int cur, const Layout& L, const Coef<R>& c, int* err,
                        cudaStream_t st, void* fout) {
-  constexpr int BX = Tile<R>::BX, NS = Tile<R>::NSLOT, MB = Tile<R>::MINB;
   if (L.i1 <= L.i0 || L.j1 <= L.j0) return;
-  dim3 grd(plan.nstrips, plan.nseg);
-  if constexpr (sizeof(R) == 4 && MRTLB_PAIR) {
-    using SM = PairSmem<BX, NS>;
-    step_pair_kernel<BX, NS, MRTLB_PAIR_MINB><<<grd, BX / 2, SM::bytes, st>>>(
-        plan.map[cur], (float*)fout, L, pair_coef(reinterpret_cast<const Coef<float>&>(c)), err, plan.seglen);
-  } else {
-    using SM = Smem<R, BX, NS>;
-    step_tiled_kernel<R, BX, NS, MB><<<grd, BX, SM::bytes, st>>>(plan.map[cur], (R*)fout, L, c, err,
-                                                                 plan.seglen);
-  }
+  const dim3 grd(plan.nstrips, plan.nseg);
+  if constexpr (sizeof(R) == 4)
+    step_pair_kernel<kPairBX, kPairSlots, kPairBlocks><<<grd, kPairBX / 2, plan.smem, st>>>(
+        plan.map[cur], (float*)fout, L, pair_coef(c), err, plan.seglen);
+  else
+    step_f64_kernel<<<grd, kRow64, plan.smem, st>>>(plan.map[cur], (double*)fout, L, c, err, plan.seglen);
 }
 
 void launch_wait_selftest(int* err, cudaStream_t st) { wait_selftest_kernel<<<1, 32, 0, st>>>(err); }

@@ -15,16 +15,15 @@
 
 namespace mrtlb {
 
-// One column strip per CTA, BX nodes wide; each CTA marches up a segment of
+// One column strip per CTA, bx nodes wide; each CTA marches up a segment of
 // rows.  Rows arrive by TMA (box = BX + 2*halo columns x 1 row x 16 planes)
 // into a ring of shared-memory slots guarded by mbarriers.
 struct TiledPlan {
   bool ok = false;
   int esize = 4;
-  int bx = 128;        // nodes per strip (threads per CTA)
-  int nslot = 6;       // ring depth
+  int bx = 128;        // nodes per strip
   int nstrips = 0, nseg = 0, seglen = 0;
-  int fill = 0;        // CTAs from which short segments march too
+  bool pays = false;   // the automatic kernel choice
   size_t smem = 0;     // dynamic shared memory per CTA
   CUtensorMap map[2];  // one per state buffer (read side; 64-byte aligned type)
 };
@@ -32,9 +31,9 @@ struct TiledPlan {
 // Encode tensor maps for both buffers and choose strips/segments; returns 0
 // on success (plan->ok set), nonzero if TMA is unavailable (plain path used).
 int plan_tiled(const Layout& L, int esize, void* f0, void* f1, TiledPlan* plan);
-// The automatic kernel choice marches segments of at least this many rows
+// The automatic FP32 choice marches segments of at least this many rows
 // whatever their number (shorter ones spend most of their time filling the
-// row pipeline), and shorter ones when there are at least `fill` of them.
+// row pipeline unless there are enough of them to fill the device).
 constexpr int kMinMarchRows = 16;
 // Choose a segment length for a target number of CTAs.
 void plan_segments(const Layout& L, int target_ctas, TiledPlan* plan);

@@ -11,8 +11,8 @@ pytestmark = pytest.mark.gpu
 
 
 @pytest.mark.parametrize("nx,ny,precision,marches", [(700, 500, "fp32", False), (1501, 300, "fp32", True),
-                                                     (1501, 701, "fp32", True), (600, 100, "fp64", False),
-                                                     (1024, 256, "fp64", True)])
+                                                     (1501, 701, "fp32", True), (100, 60, "fp64", False),
+                                                     (200, 50, "fp64", True), (1024, 256, "fp64", True)])
 def test_automatic_choice(cuda, nx, ny, precision, marches):
     cfg, fields = workloads.richtmyer_meshkov(nx=nx, ny=ny, precision=precision)
     out = {}
