@@ -49,6 +49,7 @@ __device__ __forceinline__ void load16(const R* f, long long plane, long long at
 template <typename R>
 __global__ void adj_prep_kernel(const R* __restrict__ ft, const R* __restrict__ lam, R* Ux, R* Uy, R* gsh,
                                 R* gst, Layout L, AdjCoef<R> a) {
+  after_previous();
   const int i = -1 + (int)(blockIdx.x * blockDim.x + threadIdx.x);
   const int j = -1 + (int)blockIdx.y;
   if (i > L.nx || ((i < 0 || i >= L.nx) && (j < 0 || j >= L.ny))) return;
@@ -150,6 +151,7 @@ __global__ void __launch_bounds__(128, sizeof(R) == 4 ? MRTLB_ADJ_MINB : 2)
     adj_core_kernel(const R* __restrict__ ft, const R* __restrict__ lam, const R* __restrict__ Ux,
                     const R* __restrict__ Uy, const R* __restrict__ gsh, const R* __restrict__ gst,
                     R* __restrict__ out, Layout L, AdjCoef<R> a, double* gacc, int tiles_x, int ntiles) {
+  after_previous();
   R G[16];
 #pragma unroll
   for (int k = 0; k < 16; ++k) G[k] = R(0);
@@ -185,6 +187,7 @@ template <> struct AdjTile<double> { static constexpr int BX = 64, NF = 3, NL = 
 // the whole padded grid [-1, nx] x [-1, ny].
 template <typename R>
 __global__ void adj_ghosts_kernel(R* lam, Layout L) {
+  after_previous();
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
   const int perim = 2 * L.nx + 2 * L.ny;
   if (t >= perim) return;
@@ -216,6 +219,7 @@ __global__ void adj_ghosts_kernel(R* lam, Layout L) {
 //   lambda(e)_q += [q not entering] lambda~_q + (b_q - [q not entering] a_q) / D * sum_{p entering} e_p lambda~_p.
 template <typename R>
 __global__ void adj_diffuse_kernel(R* lam, Layout L, Coef<R> c, Walls w, int side) {
+  after_previous();
   const int k = blockIdx.x * blockDim.x + threadIdx.x;
   const int n = (side < 2) ? L.ny : L.nx;
   if (k >= n) return;
@@ -253,6 +257,7 @@ __global__ void adj_diffuse_kernel(R* lam, Layout L, Coef<R> c, Walls w, int sid
 template <typename R>
 __global__ void __launch_bounds__(32) adj_walls_kernel(R* lam, const R* __restrict__ ft, Layout L, Coef<double> c, Walls w,
                                                        int side, int total) {
+  after_previous();
   int k = blockIdx.x * blockDim.x + threadIdx.x;
   if (k >= total) return;
   const int n = (side < 2) ? L.ny : L.nx;
@@ -302,13 +307,14 @@ __global__ void __launch_bounds__(32) adj_walls_kernel(R* lam, const R* __restri
 
 // Both walls of an axis in one launch, unless they share their fluid nodes.
 template <typename R>
-void launch_adj_walls(R* lam, const R* ft, const Layout& L, const Coef<double>& c, const Walls& w, cudaStream_t st) {
+void launch_adj_walls(bool early, R* lam, const R* ft, const Layout& L, const Coef<double>& c, const Walls& w,
+                      cudaStream_t st) {
   for (int s = 0; s < 4; ++s) {
     if (L.bc[s] != BC_WALL) continue;
     const int n = (s < 2) ? L.ny : L.nx, across = (s < 2) ? L.nx : L.ny;
     const bool both = (s & 1) == 0 && L.bc[s + 1] == BC_WALL && across > 3;
     const int total = both ? 2 * n : n;
-    adj_walls_kernel<R><<<(total + 31) / 32, 32, 0, st>>>(lam, ft, L, c, w, s, total);
+    launch_chained(early, adj_walls_kernel<R>, (total + 31) / 32, 32, st, lam, ft, L, c, w, s, total);
     if (both) ++s;
   }
 }
@@ -490,26 +496,30 @@ void adjoint_step(mrtlb_ctx* c, mrtlb_adjoint_state* a, long n, int li, const Co
   const R* ft = (const R*)((char*)a->seg + (size_t)n * c->state_bytes);
   const R* lam_in = (const R*)a->lam[li];
   R* lam_out = (R*)a->lam[li ^ 1];
+  // each launch of a small grid set up while the one before it runs: us per step
+  // on GB300, FP32 512 x 128 18.2 -> 12.8, 100 x 50 15.4 -> 9.7; FP64 4 x 200 54.8 ->
+  // 47.2 (above 100,000 nodes its blocks then lie unevenly)
+  const bool early = !a->march && (sizeof(R) == 4 || (long long)L.nx * L.ny <= 100000);
   if (a->march) {
     launch_adj_march<R>(a, L, a->fmap[n], a->lmap[li], lam_out, ac, c->err, rates, st);
   } else {
     dim3 g2((L.nx + 2 + 127) / 128, L.ny + 2);
-    adj_prep_kernel<R><<<g2, 128, 0, st>>>(ft, lam_in, (R*)a->ux, (R*)a->uy, (R*)a->gsh, (R*)a->gst, L, ac);
+    launch_chained(early, adj_prep_kernel<R>, g2, 128, st, ft, lam_in, (R*)a->ux, (R*)a->uy, (R*)a->gsh, (R*)a->gst, L, ac);
     const int ntiles = (int)(g2.x * g2.y);
     const int grid = std::min(ntiles, a->core_blocks);
     const bool v1 = ac.c.version == 1;  // (as the march: version 1 without the others' transposes)
     const auto core = rates ? (v1 ? adj_core_kernel<R, true, 1> : adj_core_kernel<R, true, 0>)
                             : (v1 ? adj_core_kernel<R, false, 1> : adj_core_kernel<R, false, 0>);
-    core<<<grid, 128, 0, st>>>(ft, lam_in, (const R*)a->ux, (const R*)a->uy, (const R*)a->gsh, (const R*)a->gst, lam_out,
-                               L, ac, a->gacc, (int)g2.x, ntiles);
+    launch_chained(early, core, grid, 128, st, ft, lam_in, (const R*)a->ux, (const R*)a->uy, (const R*)a->gsh,
+                   (const R*)a->gst, lam_out, L, ac, a->gacc, (int)g2.x, ntiles);
   }
   const int perim = 2 * L.nx + 2 * L.ny;
-  adj_ghosts_kernel<R><<<dim3((perim + 127) / 128, 16), 128, 0, st>>>(lam_out, L);
+  launch_chained(early, adj_ghosts_kernel<R>, dim3((perim + 127) / 128, 16), 128, st, lam_out, L);
   for (int s = 0; s < 4; ++s) {
     const int nn = (s < 2) ? L.ny : L.nx;
-    if (L.bc[s] == BC_DIFFUSE) adj_diffuse_kernel<R><<<(nn + 127) / 128, 128, 0, st>>>(lam_out, L, k, c->walls, s);
+    if (L.bc[s] == BC_DIFFUSE) launch_chained(early, adj_diffuse_kernel<R>, (nn + 127) / 128, 128, st, lam_out, L, k, c->walls, s);
   }
-  launch_adj_walls<R>(lam_out, ft, L, c->c64, c->walls, st);
+  launch_adj_walls<R>(early, lam_out, ft, L, c->c64, c->walls, st);
 }
 
 // Maps and row segments of the adjoint march; false if it cannot run.
@@ -596,7 +606,7 @@ int backward_impl(mrtlb_ctx* c, const double* dL_dmacros, const double* dL_dfK, 
     adj_dense_kernel<R><<<gd, 128, 0, st>>>(lam0, (double*)dL_dfK, L, dL_dmacros ? 2 : 0);
   }
   // walls of B^T for the seed
-  launch_adj_walls<R>(lam0, fK, L, c->c64, c->walls, st);
+  launch_adj_walls<R>(false, lam0, fK, L, c->c64, c->walls, st);
   ACK(cudaGetLastError(), "adjoint seed");
   int li = 0;  // lambda[li] holds dL/df of the latest state reached
   const long K = a->K, S = a->S;
@@ -677,11 +687,11 @@ int allocate(mrtlb_ctx* c, mrtlb_adjoint_state* a, long S, long nck) {
     }
   }
   // the fused march of the adjoint step, or the two-pass kernels: us per step on
-  // GB300, two-pass / march, FP32 512 x 128 18.2 / 21.5, 1024 x 256 31.5 / 25.6;
-  // FP64, bound by its instructions, of which the march has as many and more
-  // halo, 700 x 500 463 / 503
+  // GB300, two-pass / march, FP32 512 x 128 12.8 / 21.5, 1024 x 256 26.4 / 25.7,
+  // 700 x 500 32.7 / 29.9; FP64, bound by its instructions, of which the march
+  // has as many and more halo, 700 x 500 463 / 503
   const long long nodes = (long long)c->L.nx * c->L.ny;
-  const bool march = c->kernel == MRTLB_KERNEL_AUTO ? nodes >= (fp64 ? 450000 : 130000) : c->kernel == MRTLB_KERNEL_TILED;
+  const bool march = c->kernel == MRTLB_KERNEL_AUTO ? nodes >= (fp64 ? 450000 : 260000) : c->kernel == MRTLB_KERNEL_TILED;
   a->march = march && plan_adj_march<R>(c, a);
   return MRTLB_OK;
 }

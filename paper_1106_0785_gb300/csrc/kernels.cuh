@@ -226,13 +226,13 @@ __device__ __forceinline__ void after_previous() {
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 template <typename... P, typename... A>
-inline void launch_chained(bool early, void (*kernel)(P...), unsigned grd, unsigned blk, cudaStream_t st, A... args) {
+inline void launch_chained(bool early, void (*kernel)(P...), dim3 grd, dim3 blk, cudaStream_t st, A... args) {
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = early ? 1 : 0;
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(grd);
-  cfg.blockDim = dim3(blk);
+  cfg.gridDim = grd;
+  cfg.blockDim = blk;
   cfg.stream = st;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
