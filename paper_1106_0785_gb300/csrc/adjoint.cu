@@ -31,6 +31,7 @@
 
 #include "adjoint.cuh"
 #include "adjoint_march.cuh"
+#include "adjoint_split.cuh"
 #include "ctx.h"
 
 namespace mrtlb {
@@ -308,13 +309,18 @@ __global__ void __launch_bounds__(32) adj_walls_kernel(R* lam, const R* __restri
 // Both walls of an axis in one launch, unless they share their fluid nodes.
 template <typename R>
 void launch_adj_walls(bool early, R* lam, const R* ft, const Layout& L, const Coef<double>& c, const Walls& w,
-                      cudaStream_t st) {
+                      const AdjSplitTable<double>* tab, cudaStream_t st) {
   for (int s = 0; s < 4; ++s) {
     if (L.bc[s] != BC_WALL) continue;
     const int n = (s < 2) ? L.ny : L.nx, across = (s < 2) ? L.nx : L.ny;
     const bool both = (s & 1) == 0 && L.bc[s + 1] == BC_WALL && across > 3;
     const int total = both ? 2 * n : n;
-    launch_chained(early, adj_walls_kernel<R>, (total + 31) / 32, 32, st, lam, ft, L, c, w, s, total);
+    // (16 lanes per wall node while those are few: Couette 4 x 200, GB300, us per
+    // adjoint step 47.2 -> 37.0 in FP64, 27.5 -> 14.9 in FP32)
+    if (tab && total <= 2048)
+      launch_chained(early, adj_walls_split_kernel<R>, (total * 16 + 31) / 32, 32, st, lam, ft, L, tab, w, s, total);
+    else
+      launch_chained(early, adj_walls_kernel<R>, (total + 31) / 32, 32, st, lam, ft, L, c, w, s, total);
     if (both) ++s;
   }
 }
@@ -400,6 +406,10 @@ struct mrtlb_adjoint_state {
   void* gst = nullptr;
   void* ux = nullptr;
   void* uy = nullptr;
+  // 16 lanes per node (version 1): the tables of the walls and, on small grids
+  // without the march, of the whole step; filled by every backward pass
+  mrtlb::AdjSplitTable<double>* walls_tab = nullptr;
+  void* split_tab = nullptr;
   double* gacc = nullptr;
   int core_blocks = 1;       // resident blocks of the core kernel on the device
   size_t bytes = 0;          // device memory held in states
@@ -448,7 +458,8 @@ void release(mrtlb_adjoint_state* a) {
   if (!a) return;
   for (void* p : a->ckpt) cudaFree(p);
   a->ckpt.clear();
-  for (void* p : {a->seg, a->lam[0], a->lam[1], a->gsh, a->gst, a->ux, a->uy, (void*)a->gacc})
+  for (void* p : {a->seg, a->lam[0], a->lam[1], a->gsh, a->gst, a->ux, a->uy, (void*)a->gacc, (void*)a->walls_tab,
+                  a->split_tab})
     if (p) cudaFree(p);
   delete a;
 }
@@ -502,6 +513,12 @@ void adjoint_step(mrtlb_ctx* c, mrtlb_adjoint_state* a, long n, int li, const Co
   const bool early = !a->march && (sizeof(R) == 4 || (long long)L.nx * L.ny <= 100000);
   if (a->march) {
     launch_adj_march<R>(a, L, a->fmap[n], a->lmap[li], lam_out, ac, c->err, rates, st);
+  } else if (a->split_tab) {
+    const int threads = 16 * (L.nx + 2) * (L.ny + 2);
+    launch_chained(early, rates ? adj_split_kernel<R, true> : adj_split_kernel<R, false>,
+                   (threads + kAdjSplitThreads - 1) / kAdjSplitThreads, kAdjSplitThreads, st, ft, lam_in, lam_out, L,
+                   (const AdjSplitTable<R>*)a->split_tab, k.mod[0], k.mod[1], k.mod[2], k.mod[3], k.inv2dx, k.inv2dy,
+                   k.modified, a->gacc);
   } else {
     dim3 g2((L.nx + 2 + 127) / 128, L.ny + 2);
     launch_chained(early, adj_prep_kernel<R>, g2, 128, st, ft, lam_in, (R*)a->ux, (R*)a->uy, (R*)a->gsh, (R*)a->gst, L, ac);
@@ -519,7 +536,7 @@ void adjoint_step(mrtlb_ctx* c, mrtlb_adjoint_state* a, long n, int li, const Co
     const int nn = (s < 2) ? L.ny : L.nx;
     if (L.bc[s] == BC_DIFFUSE) launch_chained(early, adj_diffuse_kernel<R>, (nn + 127) / 128, 128, st, lam_out, L, k, c->walls, s);
   }
-  launch_adj_walls<R>(early, lam_out, ft, L, c->c64, c->walls, st);
+  launch_adj_walls<R>(early, lam_out, ft, L, c->c64, c->walls, a->walls_tab, st);
 }
 
 // Maps and row segments of the adjoint march; false if it cannot run.
@@ -573,13 +590,16 @@ const Coef<R>& coef_of(const mrtlb_ctx* c) {
 template <typename R>
 void run_segment(mrtlb_ctx* c, mrtlb_adjoint_state* a, long len, const Coef<R>& k, cudaStream_t st, R* last) {
   TraceRange trace_("adjoint_segment");
+  // the small-grid step leaves the walls it works out in the slot it reads
+  // (Couette 4 x 200 FP64, GB300: 14.9 -> 6.4 us per forward step)
+  const bool own_walls = !a->tiled && c->split;
   for (long n = 0; n < len; ++n) {
     R* fin = slot<R>(c, a, n);
-    launch_walls<R>(fin, c->L, coef_of<R>(c), c->walls, st);
     R* fout = (n + 1 < len) ? slot<R>(c, a, n + 1) : last;
+    if (!own_walls || !fout) launch_walls<R>(fin, c->L, coef_of<R>(c), c->walls, st);
     if (!fout) break;
     if (a->tiled) launch_step_tiled<R>(a->plan[n], 0, c->L, k, c->err, st, fout);
-    else launch_plain_step<R>(c, fin, fout, k, false, st);  // (the walls are in the slot)
+    else launch_plain_step<R>(c, fin, fout, k, own_walls, st, own_walls);
   }
 }
 
@@ -596,6 +616,16 @@ int backward_impl(mrtlb_ctx* c, const double* dL_dmacros, const double* dL_dfK, 
   ACK(cudaMemsetAsync(lam0, 0, sb, st), "clear");
   ACK(cudaMemsetAsync(lam1, 0, sb, st), "clear");
   ACK(cudaMemsetAsync(a->gacc, 0, kGradSlots * 16 * sizeof(double), st), "clear");
+  if (a->walls_tab) {
+    AdjSplitTable<double> t;
+    adj_split_table<double>(adj_coef<double>(c, c->c64), c->c64, &t);
+    ACK(cudaMemcpyAsync(a->walls_tab, &t, sizeof(t), cudaMemcpyHostToDevice, st), "copy lane constants");
+  }
+  if (a->split_tab) {
+    AdjSplitTable<R> t;
+    adj_split_table<R>(adj_coef<R>(c, k), c->c64, &t);
+    ACK(cudaMemcpyAsync(a->split_tab, &t, sizeof(t), cudaMemcpyHostToDevice, st), "copy lane constants");
+  }
   // seed on B(f^K)
   R* fK = (R*)c->f[c->cur];
   launch_bc<R>(fK, L, k, c->walls, st);
@@ -606,7 +636,7 @@ int backward_impl(mrtlb_ctx* c, const double* dL_dmacros, const double* dL_dfK, 
     adj_dense_kernel<R><<<gd, 128, 0, st>>>(lam0, (double*)dL_dfK, L, dL_dmacros ? 2 : 0);
   }
   // walls of B^T for the seed
-  launch_adj_walls<R>(false, lam0, fK, L, c->c64, c->walls, st);
+  launch_adj_walls<R>(false, lam0, fK, L, c->c64, c->walls, a->walls_tab, st);
   ACK(cudaGetLastError(), "adjoint seed");
   int li = 0;  // lambda[li] holds dL/df of the latest state reached
   const long K = a->K, S = a->S;
@@ -644,6 +674,13 @@ int backward_impl(mrtlb_ctx* c, const double* dL_dmacros, const double* dL_dfK, 
     }
   return MRTLB_OK;
 }
+
+// Grids up to this many nodes take 16 lanes per node: us per adjoint step on
+// GB300, two-pass / split (with the split walls both), FP64 Couette 4 x 200 37.0 /
+// 19.0, 40 x 100 36.6 / 36.2, 100 x 40 34.2 / 31.1; FP32 Couette 4 x 200 14.9 /
+// 12.1, 100 x 40 9.8 / 8.3, 100 x 79 9.7 / 10.5.
+template <typename R>
+constexpr long long kAdjSplitNodes = sizeof(R) == 8 ? 4000 : 6000;
 
 // Buffers, tensor maps and launch plans of an adjoint state with S slots
 // and nck checkpoints.
@@ -693,6 +730,11 @@ int allocate(mrtlb_ctx* c, mrtlb_adjoint_state* a, long S, long nck) {
   const long long nodes = (long long)c->L.nx * c->L.ny;
   const bool march = c->kernel == MRTLB_KERNEL_AUTO ? nodes >= (fp64 ? 450000 : 260000) : c->kernel == MRTLB_KERNEL_TILED;
   a->march = march && plan_adj_march<R>(c, a);
+  if (c->c64.version == 1) {
+    ACK(cudaMalloc((void**)&a->walls_tab, sizeof(AdjSplitTable<double>)), "cudaMalloc(lane constants)");
+    if (!a->march && nodes <= kAdjSplitNodes<R>)
+      ACK(cudaMalloc(&a->split_tab, sizeof(AdjSplitTable<R>)), "cudaMalloc(lane constants)");
+  }
   return MRTLB_OK;
 }
 

@@ -71,11 +71,13 @@ void mrtlb_adjoint_free_internal(mrtlb_ctx* c);
 
 // One step of the plain kernel choice: a velocity per lane on small grids,
 // else a thread per node.  refill: the kernel works out walls and diffuse
-// ghosts itself (else it reads them from fin).
+// ghosts itself (else it reads them from fin).  keep: on a small grid it also
+// leaves them in fin.
 template <typename R>
-inline void launch_plain_step(const mrtlb_ctx* c, const R* fin, R* fout, const Coef<R>& k, bool refill, cudaStream_t st) {
+inline void launch_plain_step(const mrtlb_ctx* c, const R* fin, R* fout, const Coef<R>& k, bool refill, cudaStream_t st,
+                              bool keep = false) {
   if (c->split && use_split<R>(c->L))
-    launch_step_split<R>(fin, fout, c->L, k, (const SplitTable<R>*)c->split, refill, c->err, st);
+    launch_step_split<R>(fin, fout, c->L, k, (const SplitTable<R>*)c->split, refill, keep, c->err, st);
   else
     launch_step_plain<R>(fin, fout, c->L, k, refill ? &c->walls : nullptr, c->err, st);
 }

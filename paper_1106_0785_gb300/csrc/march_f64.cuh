@@ -20,6 +20,7 @@
 // batch 2.71 -> 1.92.
 #pragma once
 
+#include "lanes.cuh"
 #include "march.cuh"
 
 namespace mrtlb {
@@ -27,15 +28,6 @@ namespace {
 
 constexpr int kRow64 = 64;   // columns of a strip
 constexpr int kSlot64 = 4;   // rows in flight
-
-// 1/x from the hardware's approximation by two Newton-Raphson steps, each
-// squaring its relative error; within about an ulp.
-__device__ __forceinline__ double newton_recip(double x) {
-  double r;
-  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
-  r = fma(r, fma(-x, r, 1.0), r);
-  return fma(r, fma(-x, r, 1.0), r);
-}
 
 // Macroscopic state and harmonics of a node.
 struct Node64 {
@@ -62,7 +54,7 @@ __device__ __forceinline__ void harmonics64(const double f[16], Harm<double>& h)
 __device__ __forceinline__ void node64(const double f[16], Node64& n) {
   harmonics64(f, n.h);
   conserved_h(n.h, n.rho, n.jx, n.jy, n.e);
-  n.ir = newton_recip(n.rho);
+  n.ir = split_recip(n.rho);
   n.ux = n.jx * n.ir;
   n.uy = n.jy * n.ir;
   n.t = fma(n.jy, n.uy, n.jx * n.ux);
@@ -178,7 +170,7 @@ struct March64 {
       // shells 2 and 3 count twice in j
       const bool high = l & 8;
       h = fma((kk == 0) ? 1.0 : 2.0, high ? h : o, high ? o : h);
-      const double rho = __shfl_sync(0xffffffffu, h, 0, 16), w = h * newton_recip(rho);
+      const double rho = __shfl_sync(0xffffffffu, h, 0, 16), w = h * split_recip(rho);
       if (l == 2) u[right ? BX + 1 : 0] = w;
       if (l == 3) u[(BX + 2) + (right ? BX + 1 : 0)] = w;
     }

@@ -25,30 +25,13 @@
 //
 // Walls and diffuse ghosts (REFILL) follow from the node's own moments and
 // replace the neighbour's value before its velocity is formed.
+#include "lanes.cuh"
 #include "step_split.cuh"
 
 namespace mrtlb {
 namespace {
 
 constexpr int kSplitThreads = 64;
-constexpr unsigned kAll = 0xffffffffu;
-
-template <typename R>
-__device__ __forceinline__ R from_lane(R v, int l) { return __shfl_sync(kAll, v, l, 16); }
-template <typename R>
-__device__ __forceinline__ R across(R v, int m) { return __shfl_xor_sync(kAll, v, m, 16); }
-
-// 1/x: FP32 as the other step kernels form it; FP64 by Newton-Raphson steps
-// r <- r + r (1 - x r) from the hardware's approximation, each squaring its
-// relative error (four fused multiply-adds instead of the correctly rounded
-// quotient's nine or so instructions; within about an ulp).
-__device__ __forceinline__ float split_recip(float x) { return recip(x); }
-__device__ __forceinline__ double split_recip(double x) {
-  double r;
-  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
-  r = fma(r, fma(-x, r, 1.0), r);
-  return fma(r, fma(-x, r, 1.0), r);
-}
 
 // p = rho T and t = rho |u|^2
 __device__ __forceinline__ double split_pressure(double, double jx, double jy, double e, double, double t) {
@@ -58,45 +41,11 @@ __device__ __forceinline__ float split_pressure(float rho, float jx, float jy, f
   return rho * temperature(rho, jx, jy, e, ir);  // (the compensated numerator)
 }
 
-// The lane's constants that follow from its place.
-template <typename R>
-struct Lane {
-  int l, s, k;
-  bool axis, half;  // axis: shells of axis velocities; half: an axis shell's X or Y
-  __device__ __forceinline__ explicit Lane(int lane) : l(lane & 15), s((lane & 15) >> 2), k(lane & 3) {
-    axis = (s & 1) == 0;
-    half = axis && k >= 2;
-  }
-  // f_l -> harmonic k of shell s
-  __device__ __forceinline__ R harmonic(R v) const {
-    R o = across(v, 2);
-    v = (k < 2) ? v + o : o - v;
-    o = across(v, 1);
-    if (!axis && k == 2) o = -o;
-    return v * (k == 1 ? R(-1) : R(1)) + (half ? R(0) : o);
-  }
-  // harmonic k of shell s -> the value at velocity l (pre-scaled harmonics)
-  __device__ __forceinline__ R velocity(R v) const {
-    R o = across(v, 1);
-    v = v * ((k == 1 || (k == 3 && !axis)) ? R(-1) : R(1)) + (half ? R(0) : o);
-    o = across(v, 2);
-    if (k == 1 && !axis) o = -o;
-    return v * ((k == 2 || (k == 3 && axis)) ? R(-1) : R(1)) + o;
-  }
-  // moment s of family k from harmonic k of the four shells
-  __device__ __forceinline__ R moment(R h, const R c[4]) const {
-    R m = c[0] * from_lane(h, k);
-#pragma unroll
-    for (int r = 1; r < 4; ++r) m += c[r] * from_lane(h, 4 * r + k);
-    return m;
-  }
-};
-
 template <typename R, bool REFILL>
-__global__ void __launch_bounds__(kSplitThreads) step_split_kernel(const R* __restrict__ fin, R* __restrict__ fout, const Layout L,
+__global__ void __launch_bounds__(kSplitThreads) step_split_kernel(const R* fin, R* __restrict__ fout, const Layout L,
                                                         const SplitTable<R>* __restrict__ tab, const R inv2dx,
                                                         const R inv2dy, const int version, const int modified,
-                                                        int* err) {
+                                                        R* keep, int* err) {
   const Lane<R> me(threadIdx.x);
   const int l = me.l, s = me.s, k = me.k;
   const int ni = L.i1 - L.i0;
@@ -160,23 +109,7 @@ __global__ void __launch_bounds__(kSplitThreads) step_split_kernel(const R* __re
   const R t = jx * ux + jy * uy;
   const R p = split_pressure(rho, jx, jy, e, ir, t);
 
-  // m - m^eq of the lane's moment: m - a z
-  const bool is10 = l == 8, is12 = l == 9, is13 = l == 13, is9 = l == 11;
-  const R z1 = (is10 ? e : ux) * (is10 ? e : is13 ? uy : ux);
-  const R q2 = is10 ? t : uy;
-  const R z2 = q2 * q2;
-  R z = (is9 ? R(3) : is10 ? R(-0.125) : l == 10 ? R(-3) : is13 ? R(0) : R(-1)) * (is9 ? z1 : z2) + (is9 ? -z2 : z1);
-  if (l == 5 || l == 7) z = uy;  // m5, m7
-  if (l == 6) z = ux;            // m6
-  const bool is67 = l == 6 || l == 7;
-  const R aw = (is67 ? R(1) : R(3)) * e + (is67 ? p : -t);
-  R a = R(0);
-  if (l == 1) a = rho;             // m4 = rho (ux^2 - uy^2)
-  if (l == 5 || l == 10) a = jx;   // m5 = jx uy, m8 = jx (ux^2 - 3 uy^2)
-  if (l == 11) a = jy;             // m9 = jy (3 ux^2 - uy^2)
-  if (is10) a = ir;                // m10 / 2 = (e^2 - (rho u^2)^2 / 8) / rho
-  if (is67 || is12 || is13) a = aw;  // (e + p) u; m12 / 2, m13 / 2: w / 2 = 3 e - rho u^2
-  R d = m - a * z;
+  R d = me.departure(m, rho, ir, jx, jy, e, ux, uy, t, p);
   if (version == 2 && l >= 14) {
     // m14 = rho ux (-4 + 10 T + 5 (ux^2 - uy^2)), m15 = rho uy (4 - 10 T + 5 (ux^2 - uy^2))
     const R T = p * ir, g = R(10) * T - R(4), w = R(5) * (ux * ux - uy * uy);
@@ -217,6 +150,9 @@ __global__ void __launch_bounds__(kSplitThreads) step_split_kernel(const R* __re
         const bool in = (sd & 1) ? vc < 0 : vc > 0;
         if (mine) b = in ? (R)(rw * tab->e64[sd][l]) : f;
       }
+      // (for the adjoint, which reads the state with its walls)
+      if (keep && live && mine)
+        keep[l * L.plane + L.node(i, j) + (sd == 0 ? -1 : sd == 1 ? 1 : sd == 2 ? -(long long)L.pitch : L.pitch)] = b;
     }
     neighbours();
     vn *= split_recip(from_lane(vn, 4 * s));
@@ -327,7 +263,7 @@ bool use_split(const Layout& L) {
 
 template <typename R>
 void launch_step_split(const R* fin, R* fout, const Layout& L, const Coef<R>& c, const SplitTable<R>* t, bool refill,
-                       int* err, cudaStream_t st) {
+                       bool keep, int* err, cudaStream_t st) {
   const int ni = L.i1 - L.i0, nj = L.j1 - L.j0;
   if (ni <= 0 || nj <= 0) return;
   const unsigned grd = (unsigned)(((long long)ni * nj * 16 + kSplitThreads - 1) / kSplitThreads);
@@ -335,13 +271,14 @@ void launch_step_split(const R* fin, R* fout, const Layout& L, const Coef<R>& c,
   // FP64 warps that share a sub-partition take turns, so blocks have to lie
   // evenly: set up early only up to two warps each (3200 nodes: 9.6 -> 14.5 us)
   const bool early = sizeof(R) == 4 || (long long)grd * (kSplitThreads / 32) <= 8LL * sm_count();
-  launch_chained(early, kernel, grd, kSplitThreads, st, fin, fout, L, t, c.inv2dx, c.inv2dy, c.version, c.modified, err);
+  launch_chained(early, kernel, grd, kSplitThreads, st, fin, fout, L, t, c.inv2dx, c.inv2dy, c.version, c.modified,
+                 keep ? const_cast<R*>(fin) : nullptr, err);
 }
 
 #define MRTLB_INSTANTIATE(R)                                                                                   \
   template void split_table<R>(const Coef<R>&, const Walls&, SplitTable<R>*);                                  \
   template bool use_split<R>(const Layout&);                                                                   \
-  template void launch_step_split<R>(const R*, R*, const Layout&, const Coef<R>&, const SplitTable<R>*, bool, int*, \
+  template void launch_step_split<R>(const R*, R*, const Layout&, const Coef<R>&, const SplitTable<R>*, bool, bool, int*, \
                                      cudaStream_t);
 MRTLB_INSTANTIATE(float)
 MRTLB_INSTANTIATE(double)

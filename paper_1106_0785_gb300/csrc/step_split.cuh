@@ -24,9 +24,10 @@ void split_table(const Coef<R>& c, const Walls& w, SplitTable<R>* t);
 template <typename R>
 bool use_split(const Layout& L);
 // One step; walls and diffuse ghosts are worked out beside their nodes when
-// `refill`, else read from fin.  `t`: the context's table on the device.
+// `refill` (and written to fin too when `keep`), else read from fin.  `t`: the
+// context's table on the device.
 template <typename R>
 void launch_step_split(const R* fin, R* fout, const Layout& L, const Coef<R>& c, const SplitTable<R>* t, bool refill,
-                       int* err, cudaStream_t st);
+                       bool keep, int* err, cudaStream_t st);
 
 }  // namespace mrtlb
