@@ -74,6 +74,16 @@ __device__ __forceinline__ void tma_load_row(void* dst, const CUtensorMap* map, 
       "l"((uint64_t)map), "r"(x), "r"(y), "r"(0), "r"(smem_u32(bar))
       : "memory");
 }
+// the same, the lines to leave L2 before others (a row that is read once)
+__device__ __forceinline__ void tma_load_row_once(void* dst, const CUtensorMap* map, int x, int y, uint64_t* bar) {
+  uint64_t policy;
+  asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(policy));
+  asm volatile(
+      "cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes.L2::cache_hint"
+      " [%0], [%1, {%2, %3, %4}], [%5], %6;" ::"r"(smem_u32(dst)),
+      "l"((uint64_t)map), "r"(x), "r"(y), "r"(0), "r"(smem_u32(bar)), "l"(policy)
+      : "memory");
+}
 __device__ __forceinline__ void fence_proxy_async() {
   asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
 }

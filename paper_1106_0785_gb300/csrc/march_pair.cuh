@@ -70,6 +70,7 @@ struct PairMarch {
   int* err;
   long long plane;
   int t, x, boxx, r_first, r_last, issued_to, kbase;
+  bool once = false;  // rows leave L2 first (TiledPlan::once)
   int pre = 0;  // rows of this segment already issued while the previous one ran
   bool act0, act1;
   PairGhosts pg;  // x ghosts of the segment's columns
@@ -90,7 +91,8 @@ struct PairMarch {
   __device__ __forceinline__ void issue_k(int kk, const CUtensorMap* m, int bx, int r) {
     const int s = kk & (NSLOT - 1);
     mbar_expect_tx(&bars[s], (uint32_t)SM::slot_bytes);
-    tma_load_row(slots + s * SM::SLOT, m, bx, r + 1, &bars[s]);
+    if (once) tma_load_row_once(slots + s * SM::SLOT, m, bx, r + 1, &bars[s]);
+    else tma_load_row(slots + s * SM::SLOT, m, bx, r + 1, &bars[s]);
   }
   __device__ __forceinline__ void issue(int r) { issue_k(k(r), map, boxx, r); }
   // thread 0, after a barrier: one row into the slot that just became free

@@ -54,13 +54,14 @@ __global__ void __launch_bounds__(kRow64) step_f64_kernel(const __grid_constant_
 template <int BX, int NSLOT, int MINB>
 __global__ void __launch_bounds__(BX / 2, MINB)
     step_pair_kernel(const __grid_constant__ CUtensorMap tmap, float* __restrict__ fout, const Layout L,
-                     const __grid_constant__ Coef<P2> c, int* err, const int seglen) {
+                     const __grid_constant__ Coef<P2> c, int* err, const int seglen, const bool once) {
   using SM = PairSmem<BX, NSLOT>;
   extern __shared__ __align__(128) unsigned char smem_raw[];
   const int ja = L.j0 + blockIdx.y * seglen;
   const int jb = min(ja + seglen, L.j1);
   if (ja >= jb) return;  // uniform over the CTA
   PairMarch<BX, NSLOT> m;
+  m.once = once;
   m.slots = reinterpret_cast<float*>(smem_raw);
   m.U = reinterpret_cast<float*>(smem_raw + SM::u_off);
   m.bars = reinterpret_cast<uint64_t*>(smem_raw + SM::bar_off);
@@ -218,6 +219,15 @@ int plan_tiled(const Layout& L, int esize, void* f0, void* f1, TiledPlan* plan) 
       }
     }
   }
+  // Where the two buffers together are larger than L2 and one of them fits, what a
+  // step reads should make room for what it writes, which the next one reads.
+  // GB300 (L2 129 MB), us per step without / with: 1501 x 701 (141 MB) 28.3 / 27.2,
+  // 2048 x 600 (163 MB) 28.4 / 26.7, 2048 x 700 (190 MB) 33.0 / 31.4, 2048 x 800
+  // (217 MB) 37.1 / 36.5; but 2048 x 900 (245 MB) 40.8 / 41.4, 4096 x 1024 87.1 / 98.8.
+  int l2 = 0;
+  cudaDeviceGetAttribute(&l2, cudaDevAttrL2CacheSize, dev);
+  const double both = 2.0 * 16.0 * (double)L.plane * esize;
+  plan->once = esize == 4 && both > 1.0 * l2 && both <= 1.6 * l2;
   // FP32: the CTAs with which a march of short segments (8 rows or more) beats
   // the plain kernel, measured on GB300, us per step, plain / march: 700 x 500
   // (2.5 CTAs per SM) 13.4 / 16.7, 1501 x 300 (3.0) 16.5 / 15.4, 1000 x 600
@@ -265,7 +275,7 @@ void launch_step_tiled(const TiledPlan& plan, int cur, const Layout& L, const Co
   const dim3 grd(plan.nstrips, plan.nseg);
   if constexpr (sizeof(R) == 4)
     step_pair_kernel<kPairBX, kPairSlots, kPairBlocks><<<grd, kPairBX / 2, plan.smem, st>>>(
-        plan.map[cur], (float*)fout, L, pair_coef(c), err, plan.seglen);
+        plan.map[cur], (float*)fout, L, pair_coef(c), err, plan.seglen, plan.once);
   else
     step_f64_kernel<<<grd, kRow64, plan.smem, st>>>(plan.map[cur], (double*)fout, L, c, err, plan.seglen);
 }

@@ -24,6 +24,7 @@ struct TiledPlan {
   int bx = 128;        // nodes per strip
   int nstrips = 0, nseg = 0, seglen = 0;
   bool pays = false;   // the automatic kernel choice
+  bool once = false;   // FP32: the rows that are read leave L2 before those written
   size_t smem = 0;     // dynamic shared memory per CTA
   CUtensorMap map[2];  // one per state buffer (read side; 64-byte aligned type)
 };
