@@ -48,7 +48,7 @@ struct mrtlb_ctx {
   // library-owned scratch
   int* err = nullptr;            // device error word; the start of the scratch allocation
   void* split = nullptr;         // SplitTable of the context's precision (small grids), in it
-  double* acc = nullptr;         // 5 doubles for mrtlb_reduce, in it
+  double* acc = nullptr;         // 9 doubles for mrtlb_reduce, in it
   double* Tprev = nullptr;       // [ny][nx] for the residual
   int have_prev = 0;
   void* staging = nullptr;       // dense f or 4 FP64 fields

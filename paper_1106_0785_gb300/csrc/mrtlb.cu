@@ -666,13 +666,15 @@ extern "C" int mrtlb_reduce(mrtlb_ctx* c, double out[5]) {
   if (!c->Tprev) CK(cudaMalloc((void**)&c->Tprev, n * sizeof(double)), "cudaMalloc(Tprev)");
   void* f = c->f[c->cur];
   enqueue_walls(c, f, c->stream);
-  CK(cudaMemsetAsync(c->acc, 0, 5 * sizeof(double), c->stream), "cudaMemsetAsync");
+  CK(cudaMemsetAsync(c->acc, 0, 9 * sizeof(double), c->stream), "cudaMemsetAsync");
   if (c->prec == MRTLB_FP64) launch_reduce<double>((const double*)f, c->acc, c->Tprev, c->have_prev, c->L, c->stream);
   else launch_reduce<float>((const float*)f, c->acc, c->Tprev, c->have_prev, c->L, c->stream);
   int rc = check_launch(c, "reduce");
   if (rc) return rc;
-  CK(cudaMemcpyAsync(out, c->acc, 5 * sizeof(double), cudaMemcpyDeviceToHost, c->stream), "copy sums");
+  double acc[9];  // the sums, the residual, the sums' rounding
+  CK(cudaMemcpyAsync(acc, c->acc, sizeof(acc), cudaMemcpyDeviceToHost, c->stream), "copy sums");
   rc = sync_and_check(c);
+  for (int k = 0; k < 5; ++k) out[k] = k < 4 ? acc[k] + acc[5 + k] : acc[k];
   // T_prev holds this call's temperatures unless the device work itself
   // failed (a latched non-physical state or expired wait still let it run)
   c->have_prev = (rc == MRTLB_OK || rc == MRTLB_ERR_NONPHYSICAL || rc == MRTLB_ERR_TIMEOUT) ? 1 : 0;
