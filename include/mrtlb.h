@@ -133,8 +133,9 @@ int mrtlb_init_equilibrium(mrtlb_ctx* ctx, const double* rho, const double* ux,
  * f^n (when there are walls), then advances every non-wall node
  * (Sec. II-III); the step kernel also writes the new values of edge nodes
  * into the ghost layer of f^{n+1} that mirrors them (periodic or outflow),
- * so a step costs one kernel launch, two with walls.  Asynchronous on the
- * context stream. */
+ * so a step costs one kernel launch.  Wall nodes are refilled within it on
+ * small grids and by the plain kernel; the tiled kernel has them refilled by
+ * a launch of its own before it.  Asynchronous on the context stream. */
 int mrtlb_step(mrtlb_ctx* ctx, long nsteps);
 
 /* Macroscopic fields of the current state as FP64 [ny][nx]: rho = f^_1,
@@ -175,10 +176,13 @@ int mrtlb_sync(mrtlb_ctx* ctx);
 
 /* Step kernel selection.  MRTLB_KERNEL_TILED is the TMA-fed row-marching
  * kernel (one CTA per column strip and row segment, rows streamed through a
- * shared-memory ring); MRTLB_KERNEL_PLAIN is one thread per node reading its
- * neighbours from global memory.  Both compute the same step; AUTO (the
+ * shared-memory ring); MRTLB_KERNEL_PLAIN reads the neighbours from global
+ * memory, and takes by size a kernel with one velocity per lane (small
+ * grids), one whose blocks share their nodes' velocities (FP32 without
+ * walls) or one thread per node.  All compute the same step; AUTO (the
  * default) takes the tiled kernel when its tensor maps could be built at
- * bind time.  Selecting TILED when it is unavailable gives
+ * bind time and the grid gives it enough segments to fill the device.
+ * Selecting TILED when it is unavailable gives
  * MRTLB_ERR_UNSUPPORTED. */
 #define MRTLB_KERNEL_AUTO 0
 #define MRTLB_KERNEL_PLAIN 1
@@ -207,7 +211,8 @@ int mrtlb_timing_end(mrtlb_ctx* ctx, double* kernel_ms, long* launches);
 #define MRTLB_PEAK_FP64 2
 int mrtlb_measure_peak(int kind, double* tflops);
 
-/* Kernel launches one time step enqueues (boundary fills and the step). */
+/* Kernel launches one time step enqueues: the step, and the wall refill where
+ * it is a launch of its own (walls under the tiled kernel). */
 int mrtlb_launches_per_step(const mrtlb_ctx* ctx);
 
 /* Allocation-free conservation sums.  The paper has no counterpart: this is

@@ -12,10 +12,9 @@
 //
 // Only row j-1 of the pair's columns stays in registers from one row to
 // the next: rows j and j+1 are read from their ring slots, and u, 1/rho
-// and T of each row go to a 4-row shared ring when the row arrives.  (The
-// earlier form kept rows j-1, j, j+1 and their macros in registers and
-// shifted them down after every row: 254 registers against 211 now, and
-// about 2% slower on GB300.)
+// and T of each row go to a 4-row shared ring when the row arrives.
+// (Keeping rows j-1, j, j+1 and their macros in registers and shifting them
+// down after every row measured about 2% slower on GB300.)
 #pragma once
 
 #include <cuda.h>

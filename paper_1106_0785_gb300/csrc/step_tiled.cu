@@ -47,7 +47,7 @@ __global__ void __launch_bounds__(kRow64) step_f64_kernel(const __grid_constant_
 }
 
 // FP32 with two nodes per thread (march_pair.cuh): BX columns, BX/2 threads,
-// 211 registers, four CTAs per SM.  Measured alternatives on GB300: a launch
+// 254 registers, four CTAs per SM.  Measured alternatives on GB300: a launch
 // bound of five CTAs (168 registers: three warps share an SM sub-partition's
 // register file) was 7% slower, 64-column strips with eight one-warp CTAs
 // 5% slower.
