@@ -140,15 +140,11 @@ __device__ __forceinline__ void adj_core_node(const R* __restrict__ ft, const R*
   for (int q = 0; q < 16; ++q) out[q * P + at] = lt[q];
 }
 
-#ifndef MRTLB_ADJ_MINB
-#define MRTLB_ADJ_MINB 5
-#endif
-
 // Persistent over row tiles of 128 nodes (tile t: row -1 + t / tiles_x);
 // each thread sums the rate gradients of all its nodes before the warp
 // reduction.
 template <typename R, bool RATES, int VER>
-__global__ void __launch_bounds__(128, sizeof(R) == 4 ? MRTLB_ADJ_MINB : 2)
+__global__ void __launch_bounds__(128, 2)
     adj_core_kernel(const R* __restrict__ ft, const R* __restrict__ lam, const R* __restrict__ Ux,
                     const R* __restrict__ Uy, const R* __restrict__ gsh, const R* __restrict__ gst,
                     R* __restrict__ out, Layout L, AdjCoef<R> a, double* gacc, int tiles_x, int ntiles) {
@@ -163,6 +159,125 @@ __global__ void __launch_bounds__(128, sizeof(R) == 4 ? MRTLB_ADJ_MINB : 2)
       adj_core_node<R, RATES, VER>(ft, lam, Ux, Uy, gsh, gst, out, L, a, i, j, G);
   }
   if constexpr (RATES) flush_rate_gradients<R, 128>(G, gacc);
+}
+
+// FP32, both passes in one: a block of 128 threads takes a tile of 2^w columns,
+// prepares its nodes and those of its rim into shared memory (the rim's once
+// more than needed, instead of four planes through L2 and a launch) and gathers
+// from there.  What bounds it is latency, one node's chain deep.  us per adjoint
+// step on GB300 with / without the rate gradients, two kernels -> one: 100 x 79
+// 9.5 / 8.7 -> 6.8 / 6.3, 512 x 128 12.8 / 12.0 -> 9.2 / 8.5, 1024 x 256 26.4 / 25.0
+// -> 22.2 / 19.3; version 3 15.2 / 13.2 -> 10.3 / 9.2 at 512 x 128; narrow grids
+// gain most, 4 x 2000 18.9 -> 8.9.  Four blocks per SM, 126-128
+// registers; with five 512 x 128 takes 9.8 / 8.8, with three 11.5 / 8.5.  (FP64
+// keeps the two passes: its time is its instructions, and the rim's are extra.)
+constexpr int kAdjTileBlocks = 4;
+constexpr int kAdjTileCells = (32 + 2) * (4 + 2);  // (the widest of the tiles)
+template <bool RATES, int VER>
+__global__ void __launch_bounds__(128, kAdjTileBlocks)
+    adj_tile_kernel(const float* __restrict__ ft, const float* __restrict__ lam, float* __restrict__ out, const Layout L,
+                    const __grid_constant__ AdjCoef<float> a, double* gacc, const int w) {
+  __shared__ float sux[kAdjTileCells], suy[kAdjTileCells], ssh[kAdjTileCells], sst[kAdjTileCells];
+  const Coef<float>& c = a.c;
+  const long long P = L.plane;
+  const int t = threadIdx.x, TX = 1 << w, TY = 128 >> w, SW = TX + 2;
+  const int x0 = -1 + (int)blockIdx.x * TX, y0 = -1 + (int)blockIdx.y * TY;
+  const int tx = t & (TX - 1), ty = t >> w, i = x0 + tx, j = y0 + ty;
+  // the rim's cell this thread sees to: the rows below and above, then the columns beside
+  int hx = 0, hy = 0;
+  if (t < TX) hx = t, hy = -1;
+  else if (t < 2 * TX) hx = t - TX, hy = TY;
+  else if (t < 2 * TX + TY) hx = -1, hy = t - 2 * TX;
+  else hx = TX, hy = t - 2 * TX - TY;
+  const auto held = [&](int x, int y) {  // in [-1, nx] x [-1, ny] without its corners
+    return x >= -1 && x <= L.nx && y >= -1 && y <= L.ny && !((x < 0 || x >= L.nx) && (y < 0 || y >= L.ny));
+  };
+  const bool mine = held(i, j), adv = mine && advanced<float>(L, i, j);
+  const bool rim = t < 2 * (TX + TY);
+  after_previous();
+  float g[16], lp[16], gr[16], lr[16];
+  const long long at = L.node(mine ? i : 0, mine ? j : 0);
+  load16(ft, P, at, g);
+  load16(lam, P, at, lp);
+  const int rx = x0 + hx, ry = y0 + hy;
+  const bool rheld = rim && held(rx, ry), radv = rheld && c.modified && advanced<float>(L, rx, ry);
+  if (rheld) {
+    const long long ar = L.node(rx, ry);
+    load16(ft, P, ar, gr);
+    if (radv) load16(lam, P, ar, lr);
+  }
+  // (ghost rows behind walls are never read by an advanced node and may be empty)
+  const auto prep = [&](const float f[16], const float l[16], bool strain, int k, float& ux, float& uy) {
+    float rho, jx, jy, e, sh = 0.0f, st = 0.0f;
+    conserved(f, rho, jx, jy, e);
+    const float ir = (rho > 0.0f) ? adj_inv(rho) : 0.0f;
+    ux = jx * ir;
+    uy = jy * ir;
+    if (strain) gbar_node(c, l, e - 0.5f * (jx * ux + jy * uy), ux, uy, sh, st);
+    sux[k] = ux;
+    suy[k] = uy;
+    ssh[k] = sh;
+    sst[k] = st;
+    return ir;
+  };
+  const int me = (ty + 1) * SW + tx + 1, kr = (hy + 1) * SW + hx + 1;
+  float ux, uy;
+  const float ir = prep(g, lp, adv && c.modified, me, ux, uy);
+  if (rheld) {
+    float rux, ruy;
+    prep(gr, lr, radv, kr, rux, ruy);
+  } else if (rim) {
+    sux[kr] = suy[kr] = ssh[kr] = sst[kr] = 0.0f;
+  }
+  // (a) the neighbours' Lax-Wendroff weights on p (p - e_x uses kE, p + e_x kW,
+  // p - e_y kN, p + e_y kS), on their way before the barrier
+  float nb[16];
+#pragma unroll
+  for (int q = 0; q < 16; ++q) nb[q] = 0.0f;
+  if (mine) {
+    const bool on[4] = {advanced<float>(L, i - 1, j), advanced<float>(L, i + 1, j), advanced<float>(L, i, j - 1),
+                        advanced<float>(L, i, j + 1)};
+    const long long off[4] = {-1, 1, -(long long)L.pitch, (long long)L.pitch};
+#pragma unroll
+    for (int n = 0; n < 4; ++n) {
+      if (!on[n]) continue;
+#pragma unroll
+      for (int q = 0; q < 16; ++q)
+        if ((n < 2 ? vx_of(q) : vy_of(q)) != 0) nb[q] += c.lw[q][n] * lam[q * P + at + off[n]];
+    }
+  }
+  __syncthreads();
+  float G[16];
+#pragma unroll
+  for (int k = 0; k < 16; ++k) G[k] = 0.0f;
+  if (mine) {
+    float lt[16];
+#pragma unroll
+    for (int q = 0; q < 16; ++q) lt[q] = 0.0f;
+    // (c) the modification at the neighbours, through u(p): with the
+    // collision's own u adjoint at an advanced node, else on its own
+    float uxb = 0.0f, uyb = 0.0f;
+    if (c.modified) {
+      uxb = c.inv2dx * (ssh[me - 1] - ssh[me + 1]) + c.inv2dy * (sst[me - SW] - sst[me + SW]);
+      uyb = c.inv2dx * (sst[me - 1] - sst[me + 1]) - c.inv2dy * (ssh[me - SW] - ssh[me + SW]);
+    }
+    if (adv) {
+      const float shear = (sux[me + 1] - sux[me - 1]) * c.inv2dx - (suy[me + SW] - suy[me - SW]) * c.inv2dy;
+      const float strain = (suy[me + 1] - suy[me - 1]) * c.inv2dx + (sux[me + SW] - sux[me - SW]) * c.inv2dy;
+      collision_T_node<float, RATES, VER>(a, g, lp, ux, uy, shear, strain, uxb, uyb, lt, G);
+    } else if (c.modified) {
+      velocity_T(uxb, uyb, ux, uy, ir, lt);
+    }
+#pragma unroll
+    for (int q = 0; q < 16; ++q) out[q * P + at] = lt[q] + nb[q];
+  }
+  if constexpr (RATES) flush_rate_gradients<float, 128>(G, gacc);
+}
+// The widest tile that leaves a quarter of the lanes idle at most, else the narrowest.
+int adj_tile_shift(int ni) {
+  int w = 5;
+  while (w > 3 && 4 * ni < (3 << w) * ((ni + (1 << w) - 1) >> w)) --w;
+  return w;
 }
 
 // Adjoint march shapes: 128-column strips (FP32; 64 for FP64, same box
@@ -508,7 +623,7 @@ void adjoint_step(mrtlb_ctx* c, mrtlb_adjoint_state* a, long n, int li, const Co
   const R* lam_in = (const R*)a->lam[li];
   R* lam_out = (R*)a->lam[li ^ 1];
   // each launch of a small grid set up while the one before it runs: us per step
-  // on GB300, FP32 512 x 128 18.2 -> 12.8, 100 x 50 15.4 -> 9.7; FP64 4 x 200 54.8 ->
+  // on GB300, FP32 (in two passes) 512 x 128 18.2 -> 12.8, 100 x 50 15.4 -> 9.7; FP64 4 x 200 54.8 ->
   // 47.2 (above 100,000 nodes its blocks then lie unevenly)
   const bool early = !a->march && (sizeof(R) == 4 || (long long)L.nx * L.ny <= 100000);
   if (a->march) {
@@ -519,6 +634,13 @@ void adjoint_step(mrtlb_ctx* c, mrtlb_adjoint_state* a, long n, int li, const Co
                    (threads + kAdjSplitThreads - 1) / kAdjSplitThreads, kAdjSplitThreads, st, ft, lam_in, lam_out, L,
                    (const AdjSplitTable<R>*)a->split_tab, k.mod[0], k.mod[1], k.mod[2], k.mod[3], k.inv2dx, k.inv2dy,
                    k.modified, a->gacc);
+  } else if constexpr (sizeof(R) == 4) {
+    const int w = adj_tile_shift(L.nx + 2), rows = 128 >> w;
+    const bool v1 = ac.c.version == 1;  // (as the march: version 1 without the others' transposes)
+    const auto tile = rates ? (v1 ? adj_tile_kernel<true, 1> : adj_tile_kernel<true, 0>)
+                            : (v1 ? adj_tile_kernel<false, 1> : adj_tile_kernel<false, 0>);
+    launch_chained(early, tile, dim3((L.nx + 2 + (1 << w) - 1) >> w, (L.ny + 2 + rows - 1) / rows), 128, st, ft, lam_in,
+                   lam_out, L, ac, a->gacc, w);
   } else {
     dim3 g2((L.nx + 2 + 127) / 128, L.ny + 2);
     launch_chained(early, adj_prep_kernel<R>, g2, 128, st, ft, lam_in, (R*)a->ux, (R*)a->uy, (R*)a->gsh, (R*)a->gst, L, ac);
@@ -676,11 +798,11 @@ int backward_impl(mrtlb_ctx* c, const double* dL_dmacros, const double* dL_dfK, 
 }
 
 // Grids up to this many nodes take 16 lanes per node: us per adjoint step on
-// GB300, two-pass / split (with the split walls both), FP64 Couette 4 x 200 37.0 /
-// 19.0, 40 x 100 36.6 / 36.2, 100 x 40 34.2 / 31.1; FP32 Couette 4 x 200 14.9 /
-// 12.1, 100 x 40 9.8 / 8.3, 100 x 79 9.7 / 10.5.
+// GB300, FP64 two-pass / split (with the split walls both) Couette 4 x 200 37.0 /
+// 19.0, 40 x 100 36.6 / 36.2, 100 x 40 34.2 / 31.1; FP32 tiles / split Couette
+// 4 x 200 12.3 / 12.0, 20 x 100 7.3 / 7.4, 100 x 40 6.8 / 8.3.
 template <typename R>
-constexpr long long kAdjSplitNodes = sizeof(R) == 8 ? 4000 : 6000;
+constexpr long long kAdjSplitNodes = sizeof(R) == 8 ? 4000 : 1500;
 
 // Buffers, tensor maps and launch plans of an adjoint state with S slots
 // and nck checkpoints.
@@ -701,14 +823,16 @@ int allocate(mrtlb_ctx* c, mrtlb_adjoint_state* a, long S, long nck) {
   // the fixed inflow ghosts of every slot (a step writes the other ghosts)
   for (long n = 0; n < S; ++n) launch_inflow<R>(slot<R>(c, a, n), c->L, coef_of<R>(c), c->walls, st);
   for (int b = 0; b < 2; ++b) ACK(cudaMalloc(&a->lam[b], sb), "cudaMalloc(lambda)");
-  const size_t pb = (size_t)c->L.plane * c->esize;
-  ACK(cudaMalloc(&a->gsh, pb), "cudaMalloc(gbar)");
-  ACK(cudaMalloc(&a->gst, pb), "cudaMalloc(gbar)");
-  ACK(cudaMalloc(&a->ux, pb), "cudaMalloc(u)");
-  ACK(cudaMalloc(&a->uy, pb), "cudaMalloc(u)");
-  for (void* q : {a->gsh, a->gst, a->ux, a->uy}) ACK(cudaMemsetAsync(q, 0, pb, st), "clear");
+  if constexpr (sizeof(R) == 8) {  // the planes between the two passes
+    const size_t pb = (size_t)c->L.plane * c->esize;
+    ACK(cudaMalloc(&a->gsh, pb), "cudaMalloc(gbar)");
+    ACK(cudaMalloc(&a->gst, pb), "cudaMalloc(gbar)");
+    ACK(cudaMalloc(&a->ux, pb), "cudaMalloc(u)");
+    ACK(cudaMalloc(&a->uy, pb), "cudaMalloc(u)");
+    for (void* q : {a->gsh, a->gst, a->ux, a->uy}) ACK(cudaMemsetAsync(q, 0, pb, st), "clear");
+    a->core_blocks = core_resident_blocks<R>();
+  }
   ACK(cudaMalloc((void**)&a->gacc, kGradSlots * 16 * sizeof(double)), "cudaMalloc(grad)");
-  a->core_blocks = core_resident_blocks<R>();
   // one read map per slot for the tiled step (the write side is a plain pointer)
   TiledPlan p0;
   plan_tiled(c->L, (int)c->esize, a->seg, a->seg, &p0);
@@ -723,12 +847,12 @@ int allocate(mrtlb_ctx* c, mrtlb_adjoint_state* a, long S, long nck) {
       }
     }
   }
-  // the fused march of the adjoint step, or the two-pass kernels: us per step on
-  // GB300, two-pass / march, FP32 512 x 128 12.8 / 21.5, 1024 x 256 26.4 / 25.7,
-  // 700 x 500 32.7 / 29.9; FP64, bound by its instructions, of which the march
-  // has as many and more halo, 700 x 500 463 / 503
+  // the fused march of the adjoint step, or the kernels of smaller grids: us per
+  // step on GB300, FP32 tiles / march, 512 x 128 9.2 / 21.5, 1024 x 256 22.2 / 25.7,
+  // 700 x 500 27.5 / 29.8, 800 x 500 31.4 / 29.9, 1500 x 400 44.4 / 39.5; FP64, bound by its instructions,
+  // of which the march has as many and more halo, 700 x 500 463 / 503 (two-pass)
   const long long nodes = (long long)c->L.nx * c->L.ny;
-  const bool march = c->kernel == MRTLB_KERNEL_AUTO ? nodes >= (fp64 ? 450000 : 260000) : c->kernel == MRTLB_KERNEL_TILED;
+  const bool march = c->kernel == MRTLB_KERNEL_AUTO ? nodes >= (fp64 ? 450000 : 380000) : c->kernel == MRTLB_KERNEL_TILED;
   a->march = march && plan_adj_march<R>(c, a);
   if (c->c64.version == 1) {
     ACK(cudaMalloc((void**)&a->walls_tab, sizeof(AdjSplitTable<double>)), "cudaMalloc(lane constants)");

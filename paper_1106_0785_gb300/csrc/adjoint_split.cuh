@@ -14,7 +14,7 @@
 //     lane-chosen factor with a two-term sum (LaneJacobian), summed over the
 //     lanes with the moments' adjoints;
 //   * M^T back as the forward step's M^-1: moments to shells, two butterflies.
-// Version 1; the other versions keep the two-pass kernels.
+// Version 1; the other versions keep the kernels of larger grids.
 #pragma once
 
 #include "adjoint.cuh"
