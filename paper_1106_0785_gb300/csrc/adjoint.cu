@@ -43,6 +43,17 @@ __device__ __forceinline__ void load16(const R* f, long long plane, long long at
   for (int q = 0; q < 16; ++q) g[q] = f[q * plane + at];
 }
 
+// Node t of [-1, nx] x [-1, ny] in row-major order; false for its corners and
+// past its end.  Every lane has a node whatever the grid's width: FP64
+// instructions cost a warp the same with one active lane as with 32.  us per
+// adjoint step on GB300, rows of 128 lanes / nodes in order: 4 x 2000 172 / 51, 16 x
+// 1000 101 / 56, 128 x 128 58.9 / 37.0, 400 x 40 58.6 / 36.9, 512 x 128 124 / 104.
+__device__ __forceinline__ bool padded_node(const Layout& L, int t, int& i, int& j) {
+  j = t / (L.nx + 2) - 1;
+  i = t - (j + 1) * (L.nx + 2) - 1;
+  return j <= L.ny && !((i < 0 || i >= L.nx) && (j < 0 || j >= L.ny));
+}
+
 // Pass 1, every node of [-1, nx] x [-1, ny]: the velocity u = j / rho of
 // B(f) into two planes and, at advanced nodes, the adjoints of the two
 // strain combinations of the modification (zero elsewhere):
@@ -51,9 +62,8 @@ template <typename R>
 __global__ void adj_prep_kernel(const R* __restrict__ ft, const R* __restrict__ lam, R* Ux, R* Uy, R* gsh,
                                 R* gst, Layout L, AdjCoef<R> a) {
   after_previous();
-  const int i = -1 + (int)(blockIdx.x * blockDim.x + threadIdx.x);
-  const int j = -1 + (int)blockIdx.y;
-  if (i > L.nx || ((i < 0 || i >= L.nx) && (j < 0 || j >= L.ny))) return;
+  int i, j;
+  if (!padded_node(L, (int)(blockIdx.x * blockDim.x + threadIdx.x), i, j)) return;
   const long long at = L.node(i, j);
   R g[16];
   load16(ft, L.plane, at, g);
@@ -140,22 +150,20 @@ __device__ __forceinline__ void adj_core_node(const R* __restrict__ ft, const R*
   for (int q = 0; q < 16; ++q) out[q * P + at] = lt[q];
 }
 
-// Persistent over row tiles of 128 nodes (tile t: row -1 + t / tiles_x);
-// each thread sums the rate gradients of all its nodes before the warp
-// reduction.
+// Persistent over tiles of `each` nodes, at most 128; each thread sums the rate
+// gradients of all its nodes before the warp reduction.
 template <typename R, bool RATES, int VER>
 __global__ void __launch_bounds__(128, 2)
     adj_core_kernel(const R* __restrict__ ft, const R* __restrict__ lam, const R* __restrict__ Ux,
                     const R* __restrict__ Uy, const R* __restrict__ gsh, const R* __restrict__ gst,
-                    R* __restrict__ out, Layout L, AdjCoef<R> a, double* gacc, int tiles_x, int ntiles) {
+                    R* __restrict__ out, Layout L, AdjCoef<R> a, double* gacc, int ntiles, int each) {
   after_previous();
   R G[16];
 #pragma unroll
   for (int k = 0; k < 16; ++k) G[k] = R(0);
   for (int t = blockIdx.x; t < ntiles; t += gridDim.x) {
-    const int i = -1 + (t % tiles_x) * 128 + (int)threadIdx.x;
-    const int j = -1 + t / tiles_x;
-    if (i <= L.nx && !((i < 0 || i >= L.nx) && (j < 0 || j >= L.ny)))
+    int i, j;
+    if ((int)threadIdx.x < each && padded_node(L, t * each + (int)threadIdx.x, i, j))
       adj_core_node<R, RATES, VER>(ft, lam, Ux, Uy, gsh, gst, out, L, a, i, j, G);
   }
   if constexpr (RATES) flush_rate_gradients<R, 128>(G, gacc);
@@ -642,15 +650,18 @@ void adjoint_step(mrtlb_ctx* c, mrtlb_adjoint_state* a, long n, int li, const Co
     launch_chained(early, tile, dim3((L.nx + 2 + (1 << w) - 1) >> w, (L.ny + 2 + rows - 1) / rows), 128, st, ft, lam_in,
                    lam_out, L, ac, a->gacc, w);
   } else {
-    dim3 g2((L.nx + 2 + 127) / 128, L.ny + 2);
-    launch_chained(early, adj_prep_kernel<R>, g2, 128, st, ft, lam_in, (R*)a->ux, (R*)a->uy, (R*)a->gsh, (R*)a->gst, L, ac);
-    const int ntiles = (int)(g2.x * g2.y);
+    // (fewer than four warps to an SM go one to a block, or two or three: with
+    // four an SM issues an FP64 instruction per 76 cycles and warp instead of 64:
+    // 64 x 70 36.5 us per step in blocks of four, 34.0 of one)
+    const int n = (L.nx + 2) * (L.ny + 2), warps = (n + 31) / 32, each = 32 * std::min(4, (warps + sm_count() - 1) / sm_count());
+    const int ntiles = (n + each - 1) / each;
+    launch_chained(early, adj_prep_kernel<R>, ntiles, each, st, ft, lam_in, (R*)a->ux, (R*)a->uy, (R*)a->gsh, (R*)a->gst, L, ac);
     const int grid = std::min(ntiles, a->core_blocks);
     const bool v1 = ac.c.version == 1;  // (as the march: version 1 without the others' transposes)
     const auto core = rates ? (v1 ? adj_core_kernel<R, true, 1> : adj_core_kernel<R, true, 0>)
                             : (v1 ? adj_core_kernel<R, false, 1> : adj_core_kernel<R, false, 0>);
     launch_chained(early, core, grid, 128, st, ft, lam_in, (const R*)a->ux, (const R*)a->uy, (const R*)a->gsh,
-                   (const R*)a->gst, lam_out, L, ac, a->gacc, (int)g2.x, ntiles);
+                   (const R*)a->gst, lam_out, L, ac, a->gacc, ntiles, each);
   }
   const int perim = 2 * L.nx + 2 * L.ny;
   launch_chained(early, adj_ghosts_kernel<R>, dim3((perim + 127) / 128, 16), 128, st, lam_out, L);
@@ -850,7 +861,7 @@ int allocate(mrtlb_ctx* c, mrtlb_adjoint_state* a, long S, long nck) {
   // the fused march of the adjoint step, or the kernels of smaller grids: us per
   // step on GB300, FP32 tiles / march, 512 x 128 9.2 / 21.5, 1024 x 256 22.2 / 25.7,
   // 700 x 500 27.5 / 29.8, 800 x 500 31.4 / 29.9, 1500 x 400 44.4 / 39.5; FP64, bound by its instructions,
-  // of which the march has as many and more halo, 700 x 500 463 / 503 (two-pass)
+  // of which the march has as many and more halo, 700 x 500 441 / 503 (two-pass)
   const long long nodes = (long long)c->L.nx * c->L.ny;
   const bool march = c->kernel == MRTLB_KERNEL_AUTO ? nodes >= (fp64 ? 450000 : 380000) : c->kernel == MRTLB_KERNEL_TILED;
   a->march = march && plan_adj_march<R>(c, a);
