@@ -217,6 +217,14 @@ template <typename R>
 __device__ __forceinline__ bool advanced(const Layout& L, int i, int j) {
   return i >= L.i0 && i < L.i1 && j >= L.j0 && j < L.j1;
 }
+// Whether an advanced node reads node (i, j).  Cells that none reads (ghosts
+// beside wall nodes, the rows behind them) hold what memory or an earlier run
+// left, NaN even: their part of lambda~ is not formed, as a product with their
+// zero adjoints would keep it.
+template <typename R>
+__device__ __forceinline__ bool beside_advanced(const Layout& L, int i, int j) {
+  return advanced<R>(L, i - 1, j) || advanced<R>(L, i + 1, j) || advanced<R>(L, i, j - 1) || advanced<R>(L, i, j + 1);
+}
 
 // Rows 6 and 7 of inverse_T (all the modification needs): only the X and
 // Y harmonics of fb enter them.

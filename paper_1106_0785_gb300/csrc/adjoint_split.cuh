@@ -148,8 +148,8 @@ __global__ void __launch_bounds__(kAdjSplitThreads)
   const R m = me.moment(me.harmonic(f), cm);
   const R rho = from_lane(m, 0), e = from_lane(m, 4), jx = from_lane(m, 2), jy = from_lane(m, 3);
   const R rn = from_lane(vg, 4 * s), en = from_lane(vg, 4 * s + 1), jxn = from_lane(vg, 4 * s + 2), jyn = from_lane(vg, 4 * s + 3);
-  // one reciprocal for the node (lanes k = 1) and its neighbours; empty cells
-  // (beyond the padded grid, behind walls) are never used by an advanced node
+  // one reciprocal for the node (lanes k = 1) and its neighbours; cells without
+  // an advanced node beside them (behind walls, beyond the padded grid) hold anything
   const R den = (k == 1) ? rho : rn;
   const R rec = (den > R(0)) ? split_recip(den) : R(0);
   const R ir = from_lane(rec, 1), irn = from_lane(rec, 4 * s);
@@ -200,7 +200,9 @@ __global__ void __launch_bounds__(kAdjSplitThreads)
   // lanes of the conserved moments: rho (0, 0), e (1, 0), j_x (0, 2), j_y (0, 3)
   const R acc_e = from_lane(acc, 1);
   const R mbar = (l == 4) ? acc_e : (l == 0 || l == 2 || l == 3) ? acc : mb;
-  R lt = me.velocity(me.moment(mbar, cb_)) + selfw * lp;
+  const R local = me.velocity(me.moment(mbar, cb_));
+  R lt = (adv || an[0] || an[1] || an[2] || an[3]) ? local : R(0);  // (else B(f) means nothing there: beside_advanced)
+  lt += selfw * lp;
   lt += lw[1] * ln[0];
   lt += lw[0] * ln[1];
   lt += lw[3] * ln[2];
