@@ -4,17 +4,17 @@
 // rows; rows by TMA boxes into an NSLOT ring with bounded waits), one node per
 // thread.  What bounds it is the FP64 pipe: GB300 issues an FP64 instruction
 // per 64 cycles and SM sub-partition, so loads, shared memory and registers
-// are free beside it and only the FP64 instructions count, 275 a node:
+// are free beside it and only the FP64 instructions count, 307 a node:
 //   * a row's harmonics, moments and macroscopic state are formed once, when it
 //     arrives, and carried in registers to its update an iteration later;
 //   * u of the strip's two halo columns takes the lanes of one warp, sixteen a
 //     column (a thread each would cost that warp a whole node's instructions
 //     for two lanes' sake);
 //   * m - m^eq is formed as fused multiply-adds from the moment on, the rates
-//     are folded into M^-1 (CoefFold), 1/rho is Newton's iteration;
-//   * the Lax-Wendroff increment takes the neighbours' and the node's weights
-//     (one fused multiply-add each) instead of differences; it is summed before
-//     it meets f and rounds to nothing where all five values are equal.
+//     are folded into M^-1 (CoefFold), 1/rho is Newton's iteration.
+// (The Lax-Wendroff increment from the values' own weights instead of their
+// differences would save 32 of them, but moves a uniform region by a last place
+// at larger Courant numbers: see lw_update.)
 // Before, 472 a node. GB300, ms per step: 4096 x 1024 3.18 -> 2.21, 1024 x 256
 // 0.225 -> 0.158, 600 x 100 0.076 (one thread per node) -> 0.051; 16 grids of the
 // batch 2.71 -> 1.92.
@@ -202,9 +202,9 @@ struct March64 {
       const double* s = sc + q * SM::BW + SM::HL + t;
       const double f = s[0];
       double d = -C[q];
-      if (vx_of(q) != 0) d = fma(c.lw[q][1], s[-1], fma(c.lw[q][0], s[1], d));
-      if (vy_of(q) != 0) d = fma(c.lw[q][3], fp[q], fma(c.lw[q][2], fn[q], d));
-      v[q] = f + fma(-c.lwsum[q], f, d);
+      if (vx_of(q) != 0) d = fma(c.lw[q][1], s[-1] - f, fma(c.lw[q][0], s[1] - f, d));
+      if (vy_of(q) != 0) d = fma(c.lw[q][3], fp[q] - f, fma(c.lw[q][2], fn[q] - f, d));
+      v[q] = f + d;
       if (active) out[q * L.plane] = v[q];
       fp[q] = f;
     }

@@ -63,7 +63,7 @@ __global__ void __launch_bounds__(kSplitThreads) step_split_kernel(const R* fin,
     if (REFILL) cf[r] = tab->full[r][l];
     if (r < 3) ci[r] = tab->inv[r][l];
   }
-  const R rate = tab->rate[l], mod_a = tab->mod_a[l], mod_b = tab->mod_b[l], lwsum = tab->lwsum[l];
+  const R rate = tab->rate[l], mod_a = tab->mod_a[l], mod_b = tab->mod_b[l];
   R we[4];
   double wn[4], wd[4];
   if (REFILL) {
@@ -174,18 +174,9 @@ __global__ void __launch_bounds__(kSplitThreads) step_split_kernel(const R* fin,
   h += ci[2] * from_lane(c, 12 + k);
   const R C = me.velocity(h);
 
-  // Lax-Wendroff.  FP32: differences first (a uniform region stays uniform);
-  // FP64: the weights' form, whose increment also sums before it meets f and
-  // rounds to nothing where all five values are equal.
   R inc = -C;
-  if (sizeof(R) == 4) {
 #pragma unroll
-    for (int q = 0; q < 4; ++q) inc += lw[q] * (nb[q] - f);
-  } else {
-#pragma unroll
-    for (int q = 0; q < 4; ++q) inc += lw[q] * nb[q];
-    inc -= lwsum * f;
-  }
+  for (int q = 0; q < 4; ++q) inc += lw[q] * (nb[q] - f);  // (as lw_update: a uniform region stays uniform)
   const R v = f + inc;
   if (!live) return;
   R* out = fout + L.node(i, j);
@@ -230,7 +221,6 @@ void split_table(const Coef<R>& c, const Walls& w, SplitTable<R>* t) {
     }
     t->rate[l] = c.rate[moment[s][k]];
     for (int q = 0; q < 4; ++q) t->lw[q][l] = c.lw[l][q];
-    t->lwsum[l] = c.lwsum[l];
     for (int sd = 0; sd < 4; ++sd) {
       t->e[sd][l] = (R)w.e64[sd][l];
       t->e64[sd][l] = w.e64[sd][l];

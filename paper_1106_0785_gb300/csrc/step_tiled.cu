@@ -148,7 +148,7 @@ void plan_segments(const Layout& L, int target_ctas, TiledPlan* plan) {
 // FP64: segments of the length with the least FP64 instructions on the busiest
 // SM sub-partition (its warps take turns): a segment costs its rows and the two
 // arrivals around them, and a pair of CTAs has a warp on each sub-partition.
-// Returns whether that is less than the plain kernels take: the march's 275 a
+// Returns whether that is less than the plain kernels take: the march's 307 a
 // row and lane against 508 a node with 32 nodes a warp, or 60 with two.
 static bool plan_f64(const Layout& L, int nsm, TiledPlan* plan) {
   const int nj = std::max(1, L.j1 - L.j0);
@@ -157,7 +157,7 @@ static bool plan_f64(const Layout& L, int nsm, TiledPlan* plan) {
   for (int len = 1; len <= std::min(nj, 512); ++len) {
     const long long ctas = (long long)plan->nstrips * ((nj + len - 1) / len);
     const long long turns = ((ctas + nsm - 1) / nsm + 1) / 2;
-    const long long cost = turns * (275LL * len + 110) + 40;  // (40: the first rows' latency)
+    const long long cost = turns * (307LL * len + 110) + 40;  // (40: the first rows' latency)
     if (best < 0 || cost <= best) {
       best = cost;
       plan->seglen = len;
