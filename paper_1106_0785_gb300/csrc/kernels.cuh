@@ -100,15 +100,16 @@ struct Walls {
   double ux[4], uy[4], T[4];  // per side: wall or inflow velocity and temperature
   double rho[4];              // inflow density
   // Constants of the sides, worked out once on the host in FP64: the side's
-  // equilibrium distributions at unit density (walls, diffuse, inflow) in both
-  // precisions, and for a diffuse side the weights of the edge node's f_q and
-  // the divisor in its density (diffuse_value).
+  // equilibrium at unit density as distributions (walls, diffuse, inflow) and as
+  // moments in both precisions (wall_value), and for a diffuse side the weights
+  // of the edge node's f_q and the divisor in its density (diffuse_value).
   double e64[4][16];
-  float e32[4][16];
+  double m64[4][16];
+  float m32[4][16];
   double num[4][16], den[4];
 };
-__device__ __forceinline__ double side_e(const Walls& w, int s, int q, double) { return w.e64[s][q]; }
-__device__ __forceinline__ float side_e(const Walls& w, int s, int q, float) { return w.e32[s][q]; }
+__device__ __forceinline__ double side_moment(const Walls& w, int s, int k, double) { return w.m64[s][k]; }
+__device__ __forceinline__ float side_moment(const Walls& w, int s, int k, float) { return w.m32[s][k]; }
 
 // Boundary cells refilled before every step: NEE wall nodes (ny per x side,
 // nx per y side) and diffuse-reflection ghost cells (likewise).
@@ -158,7 +159,12 @@ __device__ __forceinline__ void diffuse_value(const Walls& w, int s, const R f[1
 }
 
 // The NEE wall node on side s from its fluid neighbour's distributions g:
-// f^eq(rho, u_w, T_w) + g - f^eq(rho, u, T), the first linear in rho.
+// g + f^eq(rho, u_w, T_w) - f^eq(rho, u, T).  The difference is formed in the
+// moments, rho times the side's at unit density minus the node's, zero for the
+// density, and is small before it goes through M^-1.  (Two full states through
+// M^-1 and then subtracted round at the states' size and the same way at every
+// step.  FP32, walls at T = 1, the wall's density against the node's: off by
+// -1.4e-7 in the mean of 20,000 nodes and by 4.4e-8 rms, instead of 6e-10 and 1e-8.)
 template <typename R>
 __device__ __forceinline__ void wall_value(const Coef<R>& c, const Walls& w, int s, const R g[16], R f[16]) {
   R rho, jx, jy, e;
@@ -166,11 +172,14 @@ __device__ __forceinline__ void wall_value(const Coef<R>& c, const Walls& w, int
   const R ir = R(1) / rho;
   const R ux = jx * ir, uy = jy * ir;
   const R T = temperature(rho, jx, jy, e, ir);
-  R eqa[16], fa[16];
-  equilibrium(c, rho, ir, jx, jy, e, ux, uy, T, eqa);
-  inverse_full(c, eqa, fa);
+  R d[16], df[16];
+  equilibrium(c, rho, ir, jx, jy, e, ux, uy, T, d);
+  d[0] = R(0);
 #pragma unroll
-  for (int q = 0; q < 16; ++q) f[q] = g[q] + (rho * side_e(w, s, q, R()) - fa[q]);
+  for (int k = 1; k < 16; ++k) d[k] = rho * side_moment(w, s, k, R()) - d[k];
+  inverse_full(c, d, df);
+#pragma unroll
+  for (int q = 0; q < 16; ++q) f[q] = g[q] + df[q];
 }
 
 // What lies beyond advanced node (i, j) across side s when that side is

@@ -259,7 +259,8 @@ static void build_sides(mrtlb_ctx* c) {
     inverse_full(c->c64, eq, w.e64[s]);
     w.den[s] = 0.0;
     for (int q = 0; q < 16; ++q) {
-      w.e32[s][q] = (float)w.e64[s][q];
+      w.m64[s][q] = eq[q];
+      w.m32[s][q] = (float)eq[q];
       double a, b;
       if (c->prec == MRTLB_FP64) {
         diffuse_weights(c->c64, s, q, a, b);

@@ -64,12 +64,12 @@ __global__ void __launch_bounds__(kSplitThreads) step_split_kernel(const R* fin,
     if (r < 3) ci[r] = tab->inv[r][l];
   }
   const R rate = tab->rate[l], mod_a = tab->mod_a[l], mod_b = tab->mod_b[l];
-  R we[4];
+  R wm[4];
   double wn[4], wd[4];
   if (REFILL) {
 #pragma unroll
     for (int sd = 0; sd < 4; ++sd) {
-      we[sd] = tab->e[sd][l];
+      wm[sd] = tab->wall[sd][l];
       wn[sd] = tab->num[sd][l];
       wd[sd] = tab->inv_den[sd];
     }
@@ -125,22 +125,17 @@ __global__ void __launch_bounds__(kSplitThreads) step_split_kernel(const R* fin,
 
   if (REFILL) {
     const R eq = (l == 0 || (l >= 2 && l <= 4)) ? m : m - d;  // (rho, j_x, j_y, e are their own equilibria)
-    R fa = R(0);         // the node's equilibrium at velocity l
-    bool any_wall = false;
-#pragma unroll
-    for (int sd = 0; sd < 4; ++sd) any_wall |= L.bc[sd] == BC_WALL;
-    if (any_wall) {
-      R h = R(0);
-#pragma unroll
-      for (int r = 0; r < 4; ++r) h += cf[r] * from_lane(eq, 4 * r + k);
-      fa = me.velocity(h);
-    }
 #pragma unroll
     for (int sd = 0; sd < 4; ++sd) {
       R& b = nb[sd ^ 1];  // side order -x, +x, -y, +y; neighbours E, W, N, S
       const bool mine = beside_refilled(L, sd, i, j);
-      if (L.bc[sd] == BC_WALL) {
-        if (mine) b = f + (rho * we[sd] - fa);
+      if (L.bc[sd] == BC_WALL && __any_sync(kAll, mine)) {
+        const R dm = (l == 0) ? R(0) : rho * wm[sd] - eq;  // (see wall_value)
+        R h = R(0);
+#pragma unroll
+        for (int r = 0; r < 4; ++r) h += cf[r] * from_lane(dm, 4 * r + k);
+        const R df = me.velocity(h);
+        if (mine) b = f + df;
       } else if (L.bc[sd] == BC_DIFFUSE && __any_sync(kAll, mine)) {
         double num = wn[sd] * (double)f;
 #pragma unroll
@@ -222,7 +217,7 @@ void split_table(const Coef<R>& c, const Walls& w, SplitTable<R>* t) {
     t->rate[l] = c.rate[moment[s][k]];
     for (int q = 0; q < 4; ++q) t->lw[q][l] = c.lw[l][q];
     for (int sd = 0; sd < 4; ++sd) {
-      t->e[sd][l] = (R)w.e64[sd][l];
+      t->wall[sd][l] = (R)(w.m64[sd][moment[s][k]] * (l == 8 || l == 9 || l == 13 ? 0.5 : 1.0));
       t->e64[sd][l] = w.e64[sd][l];
       t->num[sd][l] = w.num[sd][l];
     }

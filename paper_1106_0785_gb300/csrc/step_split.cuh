@@ -14,7 +14,7 @@ struct SplitTable {
   R full[4][16];   // the lane's harmonic from the family's four moments
   R rate[16], mod_a[16], mod_b[16];
   R lw[4][16];
-  R e[4][16];      // per side: its equilibrium distributions at unit density
+  R wall[4][16];   // per side: the lane's moment of its equilibrium at unit density
   double num[4][16], e64[4][16], inv_den[4];  // per diffuse side (Walls)
 };
 template <typename R>
