@@ -13,16 +13,20 @@ __device__ __forceinline__ R from_lane(R v, int l) { return __shfl_sync(kAll, v,
 template <typename R>
 __device__ __forceinline__ R across(R v, int m) { return __shfl_xor_sync(kAll, v, m, 16); }
 
-// 1/x: FP32 as the other step kernels form it; FP64 by Newton-Raphson steps
+// 1/x: FP32 as the other step kernels form it; FP64 by two Newton-Raphson steps
 // r <- r + r (1 - x r) from the hardware's approximation, each squaring its
 // relative error (four fused multiply-adds instead of the correctly rounded
-// quotient's nine or so instructions; within about an ulp).
+// quotient's nine or so instructions; within one ulp of it).  Where the steps
+// would leave the range (zeros, infinities, NaNs, magnitudes beyond 2^+-1021)
+// the approximation stands: 1/0 = inf and 1/inf = 0 as the quotient has them.
 __device__ __forceinline__ float split_recip(float x) { return recip(x); }
 __device__ __forceinline__ double split_recip(double x) {
   double r;
   asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
-  r = fma(r, fma(-x, r, 1.0), r);
-  return fma(r, fma(-x, r, 1.0), r);
+  double n = fma(r, fma(-x, r, 1.0), r);
+  n = fma(n, fma(-x, n, 1.0), n);
+  const unsigned e = (unsigned)__double2hiint(x) & 0x7ff00000u;
+  return (e - (2u << 20) <= (2042u << 20)) ? n : r;  // biased exponents 2 .. 2044
 }
 
 // The lane's constants that follow from its place.
