@@ -64,8 +64,8 @@ __device__ __forceinline__ DF df_join(DF a, DF b) {
   const float s = two_sum(a.hi, b.hi, e);
   return DF{s, __fadd_rn(e, __fadd_rn(a.lo, b.lo))};
 }
-// Zero or a magnitude in [2^-60, 2^60]: where df_of and products of a few such
-// values stay clear of FP32's range.
+// Zero or a magnitude in [2^-60, 2^60): what df_of takes (products of such
+// values may still pass FP32's range).
 __device__ __forceinline__ bool df_fits(double x) {
   const uint32_t h = (uint32_t)__double2hiint(x) & 0x7fffffffu;
   return x == 0.0 || (h >= (uint32_t)(1023 - 60) << 20 && h < (uint32_t)(1023 + 60) << 20);

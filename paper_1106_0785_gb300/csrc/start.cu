@@ -105,6 +105,16 @@ __device__ __forceinline__ void equilibrium_df(const InverseDF& c, DF rho, DF ux
   }
 }
 
+// Whether equilibrium_df stays inside FP32's range: its largest terms are
+// rho (u^2 + T)^2 times less than 2^13, in the fields' exponents 2^(r + 2 m + 13)
+// with m the larger of T's and twice u's.  (Small terms may fall below the range:
+// what they lose is 2^-149 beside f, which is of rho's size, 2^-60 or more.)
+__device__ __forceinline__ int exponent(double x) { return ((__double2hiint(x) >> 20) & 0x7ff) - 1023; }
+__device__ __forceinline__ bool equilibrium_df_fits(double rho, double ux, double uy, double T) {
+  const int m = max(exponent(T), 2 * max(exponent(ux), exponent(uy)));
+  return df_fits(rho) && df_fits(ux) && df_fits(uy) && df_fits(T) && exponent(rho) + 2 * m <= 100;
+}
+
 template <int VER>
 __global__ void __launch_bounds__(128) init_eq_df_kernel(const double* __restrict__ rho_in, const double* __restrict__ ux_in,
                                                          const double* __restrict__ uy_in, const double* __restrict__ T_in,
@@ -117,7 +127,7 @@ __global__ void __launch_bounds__(128) init_eq_df_kernel(const double* __restric
   const long long t = (long long)j * L.nx + i;
   const double rho = rho_in[t], ux = ux_in[t], uy = uy_in[t], T = T_in[t];
   float g[16];
-  if (df_fits(rho) && df_fits(ux) && df_fits(uy) && df_fits(T)) {
+  if (equilibrium_df_fits(rho, ux, uy, T)) {
     equilibrium_df<VER>(c, df_of(rho), df_of(ux), df_of(uy), df_of(T), g);
   } else {
     double eq[16], d[16];
