@@ -134,8 +134,9 @@ int mrtlb_init_equilibrium(mrtlb_ctx* ctx, const double* rho, const double* ux,
  * (Sec. II-III); the step kernel also writes the new values of edge nodes
  * into the ghost layer of f^{n+1} that mirrors them (periodic or outflow),
  * so a step costs one kernel launch.  Wall nodes are refilled within it on
- * small grids and by the plain kernel; the tiled kernel has them refilled by
- * a launch of its own before it.  Asynchronous on the context stream. */
+ * small grids; the tiled kernel, and the plain one on larger grids with walls,
+ * have them refilled by a launch of its own before it.  Asynchronous on the
+ * context stream. */
 int mrtlb_step(mrtlb_ctx* ctx, long nsteps);
 
 /* Macroscopic fields of the current state as FP64 [ny][nx]: rho = f^_1,
@@ -212,7 +213,7 @@ int mrtlb_timing_end(mrtlb_ctx* ctx, double* kernel_ms, long* launches);
 int mrtlb_measure_peak(int kind, double* tflops);
 
 /* Kernel launches one time step enqueues: the step, and the wall refill where
- * it is a launch of its own (walls under the tiled kernel). */
+ * it is a launch of its own (mrtlb_step). */
 int mrtlb_launches_per_step(const mrtlb_ctx* ctx);
 
 /* Allocation-free conservation sums.  The paper has no counterpart: this is

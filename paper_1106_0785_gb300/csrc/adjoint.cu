@@ -844,13 +844,13 @@ int allocate(mrtlb_ctx* c, mrtlb_adjoint_state* a, long S, long nck) {
   ACK(cudaMalloc((void**)&a->gacc, kGradSlots * 16 * sizeof(double)), "cudaMalloc(grad)");
   // one read map per slot for the tiled step (the write side is a plain pointer)
   TiledPlan p0;
-  plan_tiled(c->L, (int)c->esize, a->seg, a->seg, &p0);
-  a->tiled = use_tiled(c->kernel, p0, fp64);
+  plan_tiled(c->L, c->p.eq_version, (int)c->esize, a->seg, a->seg, &p0);
+  a->tiled = use_tiled(c->kernel, p0);
   if (a->tiled) {
     a->plan.resize(S);
     for (long n = 0; n < S; ++n) {
       void* sp = slot<R>(c, a, n);
-      if (plan_tiled(c->L, (int)c->esize, sp, sp, &a->plan[n]) != 0) {
+      if (plan_tiled(c->L, c->p.eq_version, (int)c->esize, sp, sp, &a->plan[n]) != 0) {
         a->tiled = false;
         break;
       }

@@ -76,7 +76,7 @@ void mrtlb_adjoint_free_internal(mrtlb_ctx* c);
 template <typename R>
 inline void launch_plain_step(const mrtlb_ctx* c, const R* fin, R* fout, const Coef<R>& k, bool refill, cudaStream_t st,
                               bool keep = false) {
-  if (c->split && use_split<R>(c->L))
+  if (c->split && use_split<R>(c->L, k.version))
     launch_step_split<R>(fin, fout, c->L, k, (const SplitTable<R>*)c->split, refill, keep, c->err, st);
   else
     launch_step_plain<R>(fin, fout, c->L, k, refill ? &c->walls : nullptr, c->err, st);

@@ -114,6 +114,9 @@ __device__ __forceinline__ float side_moment(const Walls& w, int s, int k, float
 // Boundary cells refilled before every step: NEE wall nodes (ny per x side,
 // nx per y side) and diffuse-reflection ghost cells (likewise).
 __host__ __device__ inline bool refilled_side(int kind) { return kind == BC_WALL || kind == BC_DIFFUSE; }
+inline bool has_side(const Layout& L, int kind) {
+  return L.bc[0] == kind || L.bc[1] == kind || L.bc[2] == kind || L.bc[3] == kind;
+}
 __host__ __device__ inline int wall_count(const Layout& L) {
   int n = 0;
   for (int s = 0; s < 4; ++s)
@@ -257,6 +260,14 @@ inline int sm_count() {
   return nsm;
 }
 
+// Larger grids with walls have them refilled by a launch before the one-thread
+// kernel, whose registers then hold no wall: GB300, us per step, beside the nodes /
+// first, FP32 1000 x 250 12.1 / 12.6, 800 x 500 17.3 / 16.4, FP64 256 x 256 85.6 / 86.8,
+// 512 x 300 164 / 160.
+inline bool plain_walls_first(const Layout& L, bool fp64) {
+  return has_side(L, BC_WALL) && !has_side(L, BC_DIFFUSE) &&
+         (long long)(L.i1 - L.i0) * (L.j1 - L.j0) > (fp64 ? 100000 : 300000);
+}
 // One step by the one-thread-per-node kernel.  With `w` it works out the walls
 // and diffuse ghosts beside its nodes itself; without, it reads them from fin.
 template <typename R>

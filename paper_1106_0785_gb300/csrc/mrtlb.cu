@@ -408,7 +408,7 @@ static int refresh_split(mrtlb_ctx* c) {
 static int ensure_scratch(mrtlb_ctx* c) {
   if (c->err) return MRTLB_OK;
   const bool fp64 = c->prec == MRTLB_FP64;
-  const bool split = fp64 ? use_split<double>(c->L) : use_split<float>(c->L);
+  const bool split = fp64 ? use_split<double>(c->L, c->p.eq_version) : use_split<float>(c->L, c->p.eq_version);
   const size_t table = !split ? 0 : fp64 ? sizeof(SplitTable<double>) : sizeof(SplitTable<float>);
   char* p = nullptr;
   CK(cudaMalloc((void**)&p, 512 + table), "cudaMalloc(scratch)");
@@ -463,7 +463,7 @@ extern "C" int mrtlb_bind(mrtlb_ctx* c, void* f_a, void* f_b, size_t bytes) {
   drop_graphs(c);
   rc = refresh_split(c);
   if (rc) return rc;
-  rc = plan_tiled(c->L, (int)c->esize, c->f[0], c->f[1], &c->plan);
+  rc = plan_tiled(c->L, c->p.eq_version, (int)c->esize, c->f[0], c->f[1], &c->plan);
   if (rc) return fail(c, MRTLB_ERR_CUDA, "tensor-map set-up failed (%d)", rc);
   return MRTLB_OK;
 }
@@ -525,20 +525,25 @@ extern "C" int mrtlb_init_equilibrium(mrtlb_ctx* c, const double* rho, const dou
   return check_launch(c, "init_equilibrium");
 }
 
-// one step reading buffer `cur` (for the march the walls refilled first)
+// Whether a step has its walls refilled by a launch before it.
+static bool walls_first(const mrtlb_ctx* c) {
+  if (wall_count(c->L) == 0) return false;
+  return use_tiled(c->kernel, c->plan) || plain_walls_first(c->L, c->prec == MRTLB_FP64);
+}
+// one step reading buffer `cur`
 static void enqueue_one(mrtlb_ctx* c, int cur, cudaStream_t st, bool timed) {
-  const bool tiled = use_tiled(c->kernel, c->plan, c->prec == MRTLB_FP64);
+  const bool tiled = use_tiled(c->kernel, c->plan), first = walls_first(c);
   void* fin = c->f[cur];
   void* fout = c->f[cur ^ 1];
   // (ghosts of fin were written through by the previous step)
-  if (tiled) enqueue_walls(c, fin, st);
+  if (first) enqueue_walls(c, fin, st);
   if (timed) cudaEventRecord(c->ev[2 * c->ev_used], st);
   if (c->prec == MRTLB_FP64) {
     if (tiled) launch_step_tiled<double>(c->plan, cur, c->L, c->c64, c->err, st, fout);
-    else launch_plain_step<double>(c, (const double*)fin, (double*)fout, c->c64, true, st);
+    else launch_plain_step<double>(c, (const double*)fin, (double*)fout, c->c64, !first, st);
   } else {
     if (tiled) launch_step_tiled<float>(c->plan, cur, c->L, c->c32, c->err, st, fout);
-    else launch_plain_step<float>(c, (const float*)fin, (float*)fout, c->c32, true, st);
+    else launch_plain_step<float>(c, (const float*)fin, (float*)fout, c->c32, !first, st);
   }
   if (timed) {
     cudaEventRecord(c->ev[2 * c->ev_used + 1], st);
@@ -799,11 +804,7 @@ extern "C" int mrtlb_timing_end(mrtlb_ctx* c, double* kernel_ms, long* launches)
 
 extern "C" int mrtlb_launches_per_step(const mrtlb_ctx* c) {
   if (!c) return MRTLB_ERR_ARG;
-  int n = 1;  // the step (it writes the ghost layer through)
-  if (!use_tiled(c->kernel, c->plan, c->prec == MRTLB_FP64)) return n;  // (and works out walls itself)
-  for (int s = 0; s < 4; ++s)
-    if (refilled_side(c->L.bc[s])) { ++n; break; }  // + the wall and diffuse-ghost fill
-  return n;
+  return walls_first(c) ? 2 : 1;  // the step (it writes the ghost layer through), and the walls' refill
 }
 
 extern "C" int mrtlb_set_kernel(mrtlb_ctx* c, int which) {

@@ -5,7 +5,7 @@
 // that chain is the whole cost: GB300 issues one FP64 instruction per 64
 // cycles and SM sub-partition, however many lanes of the warp are active, and
 // the one-thread-per-node kernel spends 508 of them a node.  Spread over the
-// 16 lanes of half a warp, a node's step is 58.
+// 16 lanes of half a warp, a node's step is 61.
 //
 // Lane l = 4 s + k holds velocity l of shell s.  Two butterfly stages inside
 // the shell leave the lane with harmonic k of its shell (k = 0: S, 1: Q on the
@@ -229,20 +229,23 @@ void split_table(const Coef<R>& c, const Walls& w, SplitTable<R>* t) {
   t->mod_b[7] = c.mod[3];
 }
 
-// The lines lie where the one-thread-per-node kernel takes over, us per step on
-// GB300, 16 lanes per node / one thread: FP64 6000 nodes 15.0 / 18.5, 8000 20.8 /
-// 18.5, with walls 9500 28.0 / 25.5 (it has two nodes a warp at 58 FP64
-// instructions, the other 32 at 508, and both fill up at 608 warps); FP32, bound
-// by the length of one thread's chain, 1600 nodes 2.58 / 2.72, 3200 2.83 / 2.73,
+// The lines lie where another kernel takes over, us per step on GB300, 16 lanes per
+// node / one thread.  FP64, which takes turns of two nodes a warp at 61 FP64
+// instructions against rounds of 32 at 508 (version 1): 6000 nodes 15.6 / 18.7, 6400
+// 18.9 / 18.5, version 2 17.2 / 19.1 and 20.8 / 18.9, version 3, whose exponentials
+// it spreads over the lanes, 6800 28.2 / 29.6; with walls 7000 23.4 / 24.2, 7560 25.4 /
+// 24.2, version 3 37.2 / 47.2; diffuse 6400 20.4 / 21.6, 7200 23.7 / 21.6.  FP32, bound
+// by the length of one thread's chain, 1600 nodes 2.2 / 2.7 (tiles above the line 2.2),
 // with walls 4000 3.45 / 3.5, diffuse 9000 4.96 / 6.5.  At the start of it all
-// Sod 400 x 4 FP64 took 18.6 -> 5.5, Couette 4 x 200 FP64 28.6 -> 5.7 and FP32
+// Sod 400 x 4 FP64 took 18.6 -> 5.7, Couette 4 x 200 FP64 28.6 -> 5.9 and FP32
 // 4.8 -> 2.6, slip Couette 100 x 5 FP64 29.4 -> 5.7 and FP32 12.0 -> 3.0.
 template <typename R>
-bool use_split(const Layout& L) {
-  const bool fp64 = sizeof(R) == 8, refill = wall_count(L) > 0;
-  bool diffuse = false;
-  for (int s = 0; s < 4; ++s) diffuse |= L.bc[s] == BC_DIFFUSE;
-  const long long most = fp64 ? (refill ? 8000 : 7000) : diffuse ? 10000 : refill ? 4000 : 2000;
+bool use_split(const Layout& L, int version) {
+  const bool wall = has_side(L, BC_WALL), diffuse = has_side(L, BC_DIFFUSE);
+  const long long most = sizeof(R) == 4 ? (diffuse ? 10000 : wall ? 4000 : 2000)
+                         : wall         ? (version == 3 ? 8000 : 7300)
+                         : diffuse      ? 6500
+                                        : (version == 3 ? 7000 : 6080);
   return (long long)(L.i1 - L.i0) * (L.j1 - L.j0) <= most;
 }
 
@@ -262,7 +265,7 @@ void launch_step_split(const R* fin, R* fout, const Layout& L, const Coef<R>& c,
 
 #define MRTLB_INSTANTIATE(R)                                                                                   \
   template void split_table<R>(const Coef<R>&, const Walls&, SplitTable<R>*);                                  \
-  template bool use_split<R>(const Layout&);                                                                   \
+  template bool use_split<R>(const Layout&, int);                                                              \
   template void launch_step_split<R>(const R*, R*, const Layout&, const Coef<R>&, const SplitTable<R>*, bool, bool, int*, \
                                      cudaStream_t);
 MRTLB_INSTANTIATE(float)

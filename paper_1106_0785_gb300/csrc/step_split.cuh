@@ -22,7 +22,7 @@ void split_table(const Coef<R>& c, const Walls& w, SplitTable<R>* t);
 
 // Whether a grid is small enough for it (the lines are in step_split.cu).
 template <typename R>
-bool use_split(const Layout& L);
+bool use_split(const Layout& L, int version);
 // One step; walls and diffuse ghosts are worked out beside their nodes when
 // `refill` (and written to fin too when `keep`), else read from fin.  `t`: the
 // context's table on the device.

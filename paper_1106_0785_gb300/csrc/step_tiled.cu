@@ -8,6 +8,7 @@
 
 #include "march_f64.cuh"
 #include "march_pair.cuh"
+#include "step_split.cuh"
 #include "step_tiled.cuh"
 
 namespace mrtlb {
@@ -148,28 +149,51 @@ void plan_segments(const Layout& L, int target_ctas, TiledPlan* plan) {
 // FP64: segments of the length with the least FP64 instructions on the busiest
 // SM sub-partition (its warps take turns): a segment costs its rows and the two
 // arrivals around them, and a pair of CTAs has a warp on each sub-partition.
-// Returns whether that is less than the plain kernels take: the march's 307 a
-// row and lane against 508 a node with 32 nodes a warp, or 60 with two.
-static bool plan_f64(const Layout& L, int nsm, TiledPlan* plan) {
+// Returns whether that is less than the kernel it would replace takes, in FP64
+// instructions of an SM's four sub-partitions with a warp each (38 ns), by
+// equilibrium version: a row of the march; a round of 32 nodes on each
+// sub-partition of the one-thread kernel, which with at most two warps an SM
+// takes 0.92 of it; what refilled sides add to either, a wall launch before the
+// march and a wall's arithmetic beside the plain kernel's nodes.  GB300, us per
+// step, one thread per node / march: version 1 100 x 72 18.7 / 17.1, 160 x 120 20.9 /
+// 30.8, 84 x 328 39.0 / 43.1, 256 x 256 76.2 / 55.2; version 3 49 x 176 29.5 / 32.3,
+// 64 x 170 33.4 / 31.0, 515 x 103 96.3 / 111, 300 x 300 158 / 136; walls, version 1, 200 x
+// 50 24.6 / 27.3, version 3 47.0 / 53.6.
+static bool plan_f64(const Layout& L, int version, int nsm, TiledPlan* plan) {
   const int nj = std::max(1, L.j1 - L.j0);
   const long long n = (long long)(L.i1 - L.i0) * nj;
+  const long long row = version == 3 ? 655 : version == 2 ? 338 : 323, round = version == 3 ? 840 : version == 2 ? 520 : 508;
   long long best = -1;
   for (int len = 1; len <= std::min(nj, 512); ++len) {
     const long long ctas = (long long)plan->nstrips * ((nj + len - 1) / len);
     const long long turns = ((ctas + nsm - 1) / nsm + 1) / 2;
-    const long long cost = turns * (307LL * len + 110) + 40;  // (40: the first rows' latency)
+    const long long cost = turns * (row * len + 110) + 40;
+    // (segments of a few rows wait for their first copies in every turn)
+    if (turns > 1 && len < std::min(4, nj)) continue;
     if (best < 0 || cost <= best) {
       best = cost;
       plan->seglen = len;
     }
   }
   plan->nseg = (nj + plan->seglen - 1) / plan->seglen;
-  const long long lanes = 128LL * nsm;  // 32 lanes on each of 4 sub-partitions
-  const long long plain = 508 * ((n + lanes - 1) / lanes), split = 60 * ((16 * n + lanes - 1) / lanes);
-  return best < plain && best < split;
+  if (use_split<double>(L, version)) return false;  // (16 lanes per node: faster up to its line)
+  const long long ctas = (long long)plan->nstrips * plan->nseg, turns = ((ctas + nsm - 1) / nsm + 1) / 2;
+  long long march = turns * row * plan->seglen + (version == 3 ? 215 : 165) - (ctas <= nsm ? 40 : 0);
+  const long long lanes = 128LL * nsm, rounds = (n + lanes - 1) / lanes;
+  long long plain = 2 * n <= lanes ? round * 23 / 25 + 20 : round * rounds + 40;
+  if (has_side(L, BC_WALL)) {
+    march += version == 3 ? 550 : 230;
+    // (with the walls' registers a last round that is nearly full, of three or more, takes one more)
+    if (rounds > 2 && rounds * lanes - n < n / 32) plain += round;
+    plain += version == 3 ? 450 + 25 * rounds : 145 + 15 * rounds;
+  } else if (has_side(L, BC_DIFFUSE)) {
+    march += 140;
+    plain += 60 + 20 * rounds;
+  }
+  return march < plain;
 }
 
-int plan_tiled(const Layout& L, int esize, void* f0, void* f1, TiledPlan* plan) {
+int plan_tiled(const Layout& L, int version, int esize, void* f0, void* f1, TiledPlan* plan) {
   plan->ok = false;
   plan->esize = esize;
   EncodeFn enc = get_encode();
@@ -228,12 +252,22 @@ int plan_tiled(const Layout& L, int esize, void* f0, void* f1, TiledPlan* plan) 
   cudaDeviceGetAttribute(&l2, cudaDevAttrL2CacheSize, dev);
   const double both = 2.0 * 16.0 * (double)L.plane * esize;
   plan->once = esize == 4 && both > 1.0 * l2 && both <= 1.6 * l2;
-  // FP32: the CTAs with which a march of short segments (8 rows or more) beats
-  // the plain kernel, measured on GB300, us per step, plain / march: 700 x 500
-  // (2.5 CTAs per SM) 13.4 / 16.7, 1501 x 300 (3.0) 16.5 / 15.4, 1000 x 600
-  // (3.9) 23.1 / 16.1, 1501 x 701 (segments of 15 rows) 44.1 / 28.4.
-  if (esize == 4) plan->pays = plan->seglen >= kMinMarchRows || plan->nstrips * plan->nseg >= 3 * nsm;
-  else plan->pays = plan_f64(L, nsm, plan);
+  // FP32: a march of short segments (8 rows or more) is one wave whose time hardly
+  // depends on the grid, the plain kernel's grows with the nodes; GB300, us per step,
+  // plain / march: 1000 x 400 13.8 / 15.6, 1501 x 300 14.8 / 15.4, 1501 x 350 17.4 / 15.6;
+  // version 3, whose plain kernel does less of it again, 1501 x 320 18.3 / 19.5, 1501 x
+  // 350 20.1 / 19.2; walls, which the plain kernel works out beside its nodes or has
+  // refilled first, 1000 x 400 17.0 / 17.3, 1501 x 280 17.9 / 17.3, version 3 1501 x 300
+  // 21.5 / 22.0.
+  if (esize == 4) {
+    const long long nodes = (long long)(L.i1 - L.i0) * (L.j1 - L.j0);
+    const bool refill = wall_count(L) > 0;
+    plan->pays = plan->seglen >= kMinMarchRows ||
+                 (refill ? nodes >= (version == 3 ? 3000LL : 2700LL) * nsm
+                         : plan->nstrips * plan->nseg >= 3 * nsm && (version != 3 || nodes >= 3300LL * nsm));
+  } else {
+    plan->pays = plan_f64(L, version, nsm, plan);
+  }
   plan->ok = true;
   return 0;
 }
@@ -260,8 +294,7 @@ int encode_row_maps(const Layout& L, int esize, void* f0, void* f1, int bx, CUte
 
 bool tiled_supported(const TiledPlan& plan) { return plan.ok; }
 
-bool use_tiled(int which, const TiledPlan& plan, bool fp64) {
-  (void)fp64;
+bool use_tiled(int which, const TiledPlan& plan) {
   if (!plan.ok) return false;
   if (which == MRTLB_KERNEL_PLAIN) return false;
   if (which == MRTLB_KERNEL_TILED) return true;

@@ -31,7 +31,8 @@ struct TiledPlan {
 
 // Encode tensor maps for both buffers and choose strips/segments; returns 0
 // on success (plan->ok set), nonzero if TMA is unavailable (plain path used).
-int plan_tiled(const Layout& L, int esize, void* f0, void* f1, TiledPlan* plan);
+// version: the equilibrium's, which the automatic choice counts with.
+int plan_tiled(const Layout& L, int version, int esize, void* f0, void* f1, TiledPlan* plan);
 // The automatic FP32 choice marches segments of at least this many rows
 // whatever their number (shorter ones spend most of their time filling the
 // row pipeline unless there are enough of them to fill the device).
@@ -42,7 +43,7 @@ bool tiled_supported(const TiledPlan& plan);
 // Row tensor maps (box = bx + 2 halo columns x 1 row x 16 planes) of two
 // state buffers; returns 0 on success.
 int encode_row_maps(const Layout& L, int esize, void* f0, void* f1, int bx, CUtensorMap out[2]);
-bool use_tiled(int which, const TiledPlan& plan, bool fp64);
+bool use_tiled(int which, const TiledPlan& plan);
 
 // One kernel whose bounded wait runs out (sets ERRBIT_TIMEOUT in *err).
 void launch_wait_selftest(int* err, cudaStream_t st);
