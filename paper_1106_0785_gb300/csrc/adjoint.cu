@@ -128,7 +128,7 @@ __device__ __forceinline__ void adj_core_node(const R* __restrict__ ft, const R*
     const R shear = (Ux[aE] - Ux[aW]) * c.inv2dx - (Uy[aN] - Uy[aS]) * c.inv2dy;
     const R strain = (Uy[aE] - Uy[aW]) * c.inv2dx + (Ux[aN] - Ux[aS]) * c.inv2dy;
     collision_T_node<R, RATES, VER>(a, g, lp, ux, uy, shear, strain, uxb, uyb, lt, G);
-  } else if (c.modified && beside_advanced<R>(L, i, j)) {
+  } else if (c.modified) {
     velocity_T(uxb, uyb, ux, uy, ir, lt);
   }
   // (a) neighbours' Lax-Wendroff weights on p
@@ -271,7 +271,7 @@ __global__ void __launch_bounds__(128, kAdjTileBlocks)
       const float shear = (sux[me + 1] - sux[me - 1]) * c.inv2dx - (suy[me + SW] - suy[me - SW]) * c.inv2dy;
       const float strain = (suy[me + 1] - suy[me - 1]) * c.inv2dx + (sux[me + SW] - sux[me - SW]) * c.inv2dy;
       collision_T_node<float, RATES, VER>(a, g, lp, ux, uy, shear, strain, uxb, uyb, lt, G);
-    } else if (c.modified && beside_advanced<float>(L, i, j)) {
+    } else if (c.modified) {
       velocity_T(uxb, uyb, ux, uy, ir, lt);
     }
 #pragma unroll

@@ -217,14 +217,6 @@ template <typename R>
 __device__ __forceinline__ bool advanced(const Layout& L, int i, int j) {
   return i >= L.i0 && i < L.i1 && j >= L.j0 && j < L.j1;
 }
-// Whether an advanced node reads node (i, j).  Cells that none reads (ghosts
-// beside wall nodes, the rows behind them) hold what memory or an earlier run
-// left, NaN even: their part of lambda~ is not formed, as a product with their
-// zero adjoints would keep it.
-template <typename R>
-__device__ __forceinline__ bool beside_advanced(const Layout& L, int i, int j) {
-  return advanced<R>(L, i - 1, j) || advanced<R>(L, i + 1, j) || advanced<R>(L, i, j - 1) || advanced<R>(L, i, j + 1);
-}
 
 // Rows 6 and 7 of inverse_T (all the modification needs): only the X and
 // Y harmonics of fb enter them.
@@ -340,8 +332,12 @@ __device__ __forceinline__ void collision_T_node(const AdjCoef<R>& a, const R g[
 }
 
 // Adjoint of u = j / rho at p carried to f(p): lt_q += (ub . (v_q - u)) / rho.
+// Cells that no advanced node reads (ghosts beside wall nodes, the rows behind
+// them) hold what memory or an earlier run left, NaN even, which a product with
+// their zero ub would keep: nothing is formed there.
 template <typename R>
 __device__ __forceinline__ void velocity_T(R uxb, R uyb, R ux, R uy, R ir, R lt[16]) {
+  if (uxb == R(0) && uyb == R(0)) return;
 #pragma unroll
   for (int q = 0; q < 16; ++q) lt[q] += (uxb * (R(vx_of(q)) - ux) + uyb * (R(vy_of(q)) - uy)) * ir;
 }

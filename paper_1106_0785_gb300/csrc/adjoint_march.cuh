@@ -156,8 +156,6 @@ struct AdjMarch {
       uyb = c.inv2dx * (pc[G1 + i1 - 1] - pc[G1 + i1 + 1]) - c.inv2dy * (pp[G0 + i1] - pn[G0 + i1]);
     }
     const bool rC = row_adv(j);
-    const bool aW = colW && rC, aE = colE && rC;
-    const bool aS = colC && row_adv(j - 1), aN = colC && row_adv(j + 1);
     if (colC && rC) {
       const R* fr = frow(j);
       R g[16], lp[16];
@@ -169,10 +167,12 @@ struct AdjMarch {
       const R shear = (pc[i1 + 1] - pc[i1 - 1]) * c.inv2dx - (pn[SM::PW + i1] - pp[SM::PW + i1]) * c.inv2dy;
       const R strain = (pc[SM::PW + i1 + 1] - pc[SM::PW + i1 - 1]) * c.inv2dx + (pn[i1] - pp[i1]) * c.inv2dy;
       collision_T_node<R, RATES, VER>(a, g, lp, ux, uy, shear, strain, uxb, uyb, lt, G);
-    } else if (c.modified && (aW || aE || aS || aN)) {  // (else B(f) means nothing there: beside_advanced)
+    } else if (c.modified) {
       velocity_T(uxb, uyb, ux, uy, pc[4 * SM::PW + i1], lt);
     }
     // neighbours' Lax-Wendroff weights: r = p - e_x (k_E), p + e_x (k_W), p - e_y (k_N), p + e_y (k_S)
+    const bool aW = colW && rC, aE = colE && rC;
+    const bool aS = colC && row_adv(j - 1), aN = colC && row_adv(j + 1);
 #pragma unroll
     for (int q = 0; q < 16; ++q) {
       if (vx_of(q) != 0) {

@@ -201,7 +201,7 @@ __global__ void __launch_bounds__(kAdjSplitThreads)
   const R acc_e = from_lane(acc, 1);
   const R mbar = (l == 4) ? acc_e : (l == 0 || l == 2 || l == 3) ? acc : mb;
   const R local = me.velocity(me.moment(mbar, cb_));
-  R lt = (adv || an[0] || an[1] || an[2] || an[3]) ? local : R(0);  // (else B(f) means nothing there: beside_advanced)
+  R lt = (adv || an[0] || an[1] || an[2] || an[3]) ? local : R(0);  // (else B(f) means nothing there: velocity_T)
   lt += selfw * lp;
   lt += lw[1] * ln[0];
   lt += lw[0] * ln[1];
