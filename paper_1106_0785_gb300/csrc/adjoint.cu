@@ -54,80 +54,78 @@ __device__ __forceinline__ bool padded_node(const Layout& L, int t, int& i, int&
   return j <= L.ny && !((i < 0 || i >= L.nx) && (j < 0 || j >= L.ny));
 }
 
-// Pass 1, every node of [-1, nx] x [-1, ny]: the velocity u = j / rho of
+// FP64 in two passes.  Pass 1, every node of [-1, nx] x [-1, ny]: the velocity u = j / rho of
 // B(f) into two planes and, at advanced nodes, the adjoints of the two
 // strain combinations of the modification (zero elsewhere):
 //   gbar_shear  = dL/d(du_x/dx - du_y/dy),  gbar_strain = dL/d(du_y/dx + du_x/dy).
-template <typename R>
-__global__ void adj_prep_kernel(const R* __restrict__ ft, const R* __restrict__ lam, R* Ux, R* Uy, R* gsh,
-                                R* gst, Layout L, AdjCoef<R> a) {
+__global__ void adj_prep_kernel(const double* __restrict__ ft, const double* __restrict__ lam, double* Ux, double* Uy, double* gsh,
+                                double* gst, Layout L, AdjCoef<double> a) {
   after_previous();
   int i, j;
   if (!padded_node(L, (int)(blockIdx.x * blockDim.x + threadIdx.x), i, j)) return;
   const long long at = L.node(i, j);
-  R g[16];
+  double g[16];
   load16(ft, L.plane, at, g);
-  R rho, jx, jy, e;
+  double rho, jx, jy, e;
   conserved(g, rho, jx, jy, e);
-  const R ir = (rho > R(0)) ? adj_inv(rho) : R(0);
-  const R ux = jx * ir, uy = jy * ir;
+  const double ir = (rho > 0.0) ? adj_inv(rho) : 0.0;
+  const double ux = jx * ir, uy = jy * ir;
   Ux[at] = ux;
   Uy[at] = uy;
-  if (!advanced<R>(L, i, j) || !a.c.modified) {
-    gsh[at] = R(0);
-    gst[at] = R(0);
+  if (!advanced<double>(L, i, j) || !a.c.modified) {
+    gsh[at] = 0.0;
+    gst[at] = 0.0;
     return;
   }
-  R lb[16];
+  double lb[16];
   load16(lam, L.plane, at, lb);
-  R sh, sn;
-  gbar_node(a.c, lb, e - R(0.5) * (jx * ux + jy * uy), ux, uy, sh, sn);
+  double sh, sn;
+  gbar_node(a.c, lb, e - 0.5 * (jx * ux + jy * uy), ux, uy, sh, sn);
   gsh[at] = sh;
   gst[at] = sn;
 }
 
-template <typename R>
-__device__ __forceinline__ R gbar_at(const R* gb, const Layout& L, int i, int j) {
-  if (i < -1 || i > L.nx || j < -1 || j > L.ny) return R(0);
+__device__ __forceinline__ double gbar_at(const double* gb, const Layout& L, int i, int j) {
+  if (i < -1 || i > L.nx || j < -1 || j > L.ny) return 0.0;
   return gb[L.node(i, j)];
 }
 
 // Pass 2: lambda~(p) for one node p of [-1, nx] x [-1, ny] (corners
 // excluded); the rate gradients of an advanced node are added to G.
-template <typename R, bool RATES, int VER>
-__device__ __forceinline__ void adj_core_node(const R* __restrict__ ft, const R* __restrict__ lam,
-                                              const R* __restrict__ Ux, const R* __restrict__ Uy,
-                                              const R* __restrict__ gsh, const R* __restrict__ gst,
-                                              R* __restrict__ out, const Layout& L, const AdjCoef<R>& a, int i,
-                                              int j, R G[16]) {
-  const Coef<R>& c = a.c;
+template <bool RATES, int VER>
+__device__ __forceinline__ void adj_core_node(const double* __restrict__ ft, const double* __restrict__ lam,
+                                              const double* __restrict__ Ux, const double* __restrict__ Uy,
+                                              const double* __restrict__ gsh, const double* __restrict__ gst,
+                                              double* __restrict__ out, const Layout& L, const AdjCoef<double>& a, int i,
+                                              int j, double G[16]) {
+  const Coef<double>& c = a.c;
   const long long P = L.plane;
   const long long at = L.node(i, j);
-  const R ux = Ux[at], uy = Uy[at];
-  R g[16], lt[16];
+  const double ux = Ux[at], uy = Uy[at];
+  double g[16], lt[16];
   load16(ft, P, at, g);
-  R rho = R(0);
+  double rho = 0.0;
 #pragma unroll
   for (int q = 0; q < 16; ++q) rho += g[q];
-  const R ir = (rho > R(0)) ? adj_inv(rho) : R(0);
+  const double ir = (rho > 0.0) ? adj_inv(rho) : 0.0;
 #pragma unroll
-  for (int q = 0; q < 16; ++q) lt[q] = R(0);
+  for (int q = 0; q < 16; ++q) lt[q] = 0.0;
   // (c) the modification at the neighbours, through u(p): with the
   // collision's own u adjoint at an advanced node, else on its own
-  R uxb = R(0), uyb = R(0);
+  double uxb = 0.0, uyb = 0.0;
   if (c.modified) {
     uxb = c.inv2dx * (gbar_at(gsh, L, i - 1, j) - gbar_at(gsh, L, i + 1, j)) +
           c.inv2dy * (gbar_at(gst, L, i, j - 1) - gbar_at(gst, L, i, j + 1));
     uyb = c.inv2dx * (gbar_at(gst, L, i - 1, j) - gbar_at(gst, L, i + 1, j)) -
           c.inv2dy * (gbar_at(gsh, L, i, j - 1) - gbar_at(gsh, L, i, j + 1));
   }
-  if (advanced<R>(L, i, j)) {
-    R lp[16];
+  if (advanced<double>(L, i, j)) {
+    double lp[16];
     load16(lam, P, at, lp);
     const long long aE = at + 1, aW = at - 1, aN = at + L.pitch, aS = at - L.pitch;
-    const R shear = (Ux[aE] - Ux[aW]) * c.inv2dx - (Uy[aN] - Uy[aS]) * c.inv2dy;
-    const R strain = (Uy[aE] - Uy[aW]) * c.inv2dx + (Ux[aN] - Ux[aS]) * c.inv2dy;
-    collision_T_node<R, RATES, VER>(a, g, lp, ux, uy, shear, strain, uxb, uyb, lt, G);
+    const double shear = (Ux[aE] - Ux[aW]) * c.inv2dx - (Uy[aN] - Uy[aS]) * c.inv2dy;
+    const double strain = (Uy[aE] - Uy[aW]) * c.inv2dx + (Ux[aN] - Ux[aS]) * c.inv2dy;
+    collision_T_node<double, RATES, VER>(a, g, lp, ux, uy, shear, strain, uxb, uyb, lt, G);
   } else if (c.modified) {
     velocity_T(uxb, uyb, ux, uy, ir, lt);
   }
@@ -136,7 +134,7 @@ __device__ __forceinline__ void adj_core_node(const R* __restrict__ ft, const R*
   const int nbj[4] = {j, j, j - 1, j + 1};
 #pragma unroll
   for (int n = 0; n < 4; ++n) {
-    if (!advanced<R>(L, nbi[n], nbj[n])) continue;
+    if (!advanced<double>(L, nbi[n], nbj[n])) continue;
     const long long ar = L.node(nbi[n], nbj[n]);
 #pragma unroll
     for (int q = 0; q < 16; ++q) {
@@ -151,21 +149,21 @@ __device__ __forceinline__ void adj_core_node(const R* __restrict__ ft, const R*
 
 // Persistent over tiles of `each` nodes, at most 128; each thread sums the rate
 // gradients of all its nodes before the warp reduction.
-template <typename R, bool RATES, int VER>
+template <bool RATES, int VER>
 __global__ void __launch_bounds__(128, 2)
-    adj_core_kernel(const R* __restrict__ ft, const R* __restrict__ lam, const R* __restrict__ Ux,
-                    const R* __restrict__ Uy, const R* __restrict__ gsh, const R* __restrict__ gst,
-                    R* __restrict__ out, Layout L, AdjCoef<R> a, double* gacc, int ntiles, int each) {
+    adj_core_kernel(const double* __restrict__ ft, const double* __restrict__ lam, const double* __restrict__ Ux,
+                    const double* __restrict__ Uy, const double* __restrict__ gsh, const double* __restrict__ gst,
+                    double* __restrict__ out, Layout L, AdjCoef<double> a, double* gacc, int ntiles, int each) {
   after_previous();
-  R G[16];
+  double G[16];
 #pragma unroll
-  for (int k = 0; k < 16; ++k) G[k] = R(0);
+  for (int k = 0; k < 16; ++k) G[k] = 0.0;
   for (int t = blockIdx.x; t < ntiles; t += gridDim.x) {
     int i, j;
     if ((int)threadIdx.x < each && padded_node(L, t * each + (int)threadIdx.x, i, j))
-      adj_core_node<R, RATES, VER>(ft, lam, Ux, Uy, gsh, gst, out, L, a, i, j, G);
+      adj_core_node<RATES, VER>(ft, lam, Ux, Uy, gsh, gst, out, L, a, i, j, G);
   }
-  if constexpr (RATES) flush_rate_gradients<R, 128>(G, gacc);
+  if constexpr (RATES) flush_rate_gradients<double, 128>(G, gacc);
 }
 
 // FP32, both passes in one: a block of 128 threads takes a tile of 2^w columns,
@@ -290,17 +288,8 @@ int adj_tile_shift(int ni) {
 // bytes), 3 B(f) slots and 4 lambda slots: about 71 KB of shared memory,
 // three CTAs per SM (measured on GB300 against 4+6, 4+4 slots and 64-,
 // 96-, 256-column strips).
-#ifndef MRTLB_ADJ_BX
-#define MRTLB_ADJ_BX 128
-#endif
-#ifndef MRTLB_ADJ_NF
-#define MRTLB_ADJ_NF 3
-#endif
-#ifndef MRTLB_ADJ_NL
-#define MRTLB_ADJ_NL 4
-#endif
 template <typename R> struct AdjTile;
-template <> struct AdjTile<float> { static constexpr int BX = MRTLB_ADJ_BX, NF = MRTLB_ADJ_NF, NL = MRTLB_ADJ_NL; };
+template <> struct AdjTile<float> { static constexpr int BX = 128, NF = 3, NL = 4; };
 template <> struct AdjTile<double> { static constexpr int BX = 64, NF = 3, NL = 4; };
 
 // B^T, ghosts: every edge node collects the adjoints of the ghost cells that
@@ -337,7 +326,7 @@ __global__ void adj_ghosts_kernel(R* lam, Layout L) {
 }
 
 // B^T, diffuse reflection on side s: the ghost beyond edge node e holds
-// g = P f(e) with P linear (diffuse_ghost), so lambda(e) += P^T lambda~(g):
+// g = P f(e) with P linear (diffuse_value), so lambda(e) += P^T lambda~(g):
 //   lambda(e)_q += [q not entering] lambda~_q + (b_q - [q not entering] a_q) / D * sum_{p entering} e_p lambda~_p.
 template <typename R>
 __global__ void adj_diffuse_kernel(R* lam, Layout L, Coef<R> c, Walls w, int side) {
@@ -548,17 +537,12 @@ struct mrtlb_adjoint_state {
 namespace {
 
 // Blocks of the core kernel that fit on the device at once (its persistent grid).
-template <typename R>
 int core_resident_blocks() {
-#if defined(MRTLB_ADJ_PERSIST) && MRTLB_ADJ_PERSIST == 0
-  return 1 << 30;
-#else
   int dev = 0, nsm = 1, per = 1;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, adj_core_kernel<R, true, 0>, 128, 0);
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, adj_core_kernel<true, 0>, 128, 0);
   return std::max(1, nsm) * std::max(1, per);
-#endif
 }
 
 int afail(mrtlb_ctx* c, int code, const char* msg) {
@@ -653,11 +637,11 @@ void adjoint_step(mrtlb_ctx* c, mrtlb_adjoint_state* a, long n, int li, const Co
     // 64 x 70 36.5 us per step in blocks of four, 34.0 of one)
     const int n = (L.nx + 2) * (L.ny + 2), warps = (n + 31) / 32, each = 32 * std::min(4, (warps + sm_count() - 1) / sm_count());
     const int ntiles = (n + each - 1) / each;
-    launch_chained(early, adj_prep_kernel<R>, ntiles, each, st, ft, lam_in, (R*)a->ux, (R*)a->uy, (R*)a->gsh, (R*)a->gst, L, ac);
+    launch_chained(early, adj_prep_kernel, ntiles, each, st, ft, lam_in, (R*)a->ux, (R*)a->uy, (R*)a->gsh, (R*)a->gst, L, ac);
     const int grid = std::min(ntiles, a->core_blocks);
     const bool v1 = ac.c.version == 1;  // (as the march: version 1 without the others' transposes)
-    const auto core = rates ? (v1 ? adj_core_kernel<R, true, 1> : adj_core_kernel<R, true, 0>)
-                            : (v1 ? adj_core_kernel<R, false, 1> : adj_core_kernel<R, false, 0>);
+    const auto core = rates ? (v1 ? adj_core_kernel<true, 1> : adj_core_kernel<true, 0>)
+                            : (v1 ? adj_core_kernel<false, 1> : adj_core_kernel<false, 0>);
     launch_chained(early, core, grid, 128, st, ft, lam_in, (const R*)a->ux, (const R*)a->uy, (const R*)a->gsh,
                    (const R*)a->gst, lam_out, L, ac, a->gacc, ntiles, each);
   }
@@ -839,7 +823,7 @@ int allocate(mrtlb_ctx* c, mrtlb_adjoint_state* a, long S, long nck) {
     ACK(cudaMalloc(&a->ux, pb), "cudaMalloc(u)");
     ACK(cudaMalloc(&a->uy, pb), "cudaMalloc(u)");
     for (void* q : {a->gsh, a->gst, a->ux, a->uy}) ACK(cudaMemsetAsync(q, 0, pb, st), "clear");
-    a->core_blocks = core_resident_blocks<R>();
+    a->core_blocks = core_resident_blocks();
   }
   ACK(cudaMalloc((void**)&a->gacc, kGradSlots * 16 * sizeof(double)), "cudaMalloc(grad)");
   // one read map per slot for the tiled step (the write side is a plain pointer)

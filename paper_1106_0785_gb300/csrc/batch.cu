@@ -90,10 +90,6 @@ __global__ void __launch_bounds__(kRow64) step_batched_f64_kernel(const BatchIns
   }
 }
 
-#ifndef MRTLB_BATCH_PREFETCH
-#define MRTLB_BATCH_PREFETCH 1
-#endif
-
 // FP32 with two nodes per thread (march_pair.cuh): BX/2 threads per CTA;
 // each tile's coefficients are expanded into pairs as they are copied.
 template <int BX, int NSLOT>
@@ -153,7 +149,7 @@ __global__ void __launch_bounds__(BX / 2, MINB)
     m.fout = in->f[cur ^ 1];
     __syncthreads();  // coefficients in place (and the previous tile done with them); next_tile set
     const int nti = next_tile;
-    if (MRTLB_BATCH_PREFETCH && nti < ntiles) {  // the next tile streams in behind this one
+    if (nti < ntiles) {  // the next tile streams in behind this one
       const int4 nt = tiles[nti];
       const BatchInst<float>* nin = insts + nt.x;
       m.set_next(&nin->map[cur], nin->L.xoff + nt.y - SM::HL, nt.z, nt.w);
