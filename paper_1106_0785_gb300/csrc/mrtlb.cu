@@ -680,7 +680,8 @@ extern "C" int mrtlb_reduce(mrtlb_ctx* c, double out[5]) {
   double acc[9];  // the sums, the residual, the sums' rounding
   CK(cudaMemcpyAsync(acc, c->acc, sizeof(acc), cudaMemcpyDeviceToHost, c->stream), "copy sums");
   rc = sync_and_check(c);
-  for (int k = 0; k < 5; ++k) out[k] = k < 4 ? acc[k] + acc[5 + k] : acc[k];
+  if (rc != MRTLB_ERR_CUDA)  // (the copy may not have been made)
+    for (int k = 0; k < 5; ++k) out[k] = k < 4 ? acc[k] + acc[5 + k] : acc[k];
   // T_prev holds this call's temperatures unless the device work itself
   // failed (a latched non-physical state or expired wait still let it run)
   c->have_prev = (rc == MRTLB_OK || rc == MRTLB_ERR_NONPHYSICAL || rc == MRTLB_ERR_TIMEOUT) ? 1 : 0;
