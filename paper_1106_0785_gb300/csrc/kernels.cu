@@ -12,7 +12,7 @@ namespace mrtlb {
 // REFILL: walls and diffuse ghosts are functions of the node beside them, so
 // the node works them out from its own distributions and a step needs no
 // launch before it that refills them in memory (whoever reads them there
-// refills them first).
+// refills them first; and so do larger grids with walls, plain_walls_first).
 // ---------------------------------------------------------------------------
 template <typename R>
 __device__ __forceinline__ void velocity(const R g[16], R& ux, R& uy) {

@@ -15,9 +15,9 @@
 // (The Lax-Wendroff increment from the values' own weights instead of their
 // differences would save 32 of them, but moves a uniform region by a last place
 // at larger Courant numbers: see lw_update.)
-// Before, 472 a node. GB300, ms per step: 4096 x 1024 3.18 -> 2.21, 1024 x 256
-// 0.225 -> 0.158, 600 x 100 0.076 (one thread per node) -> 0.051; 16 grids of the
-// batch 2.71 -> 1.92.
+// Before, 472 a node. GB300, ms per step: 4096 x 1024 3.18 -> 2.46, 1024 x 256
+// 0.225 -> 0.177, 600 x 100 0.076 (one thread per node) -> 0.055; 16 grids of the
+// batch 2.71 -> 2.14.
 #pragma once
 
 #include "lanes.cuh"

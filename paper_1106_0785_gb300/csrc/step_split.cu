@@ -237,8 +237,8 @@ void split_table(const Coef<R>& c, const Walls& w, SplitTable<R>* t) {
 // 24.2, version 3 37.2 / 47.2; diffuse 6400 20.4 / 21.6, 7200 23.7 / 21.6.  FP32, bound
 // by the length of one thread's chain, 1600 nodes 2.2 / 2.7 (tiles above the line 2.2),
 // with walls 4000 3.45 / 3.5, diffuse 9000 4.96 / 6.5.  At the start of it all
-// Sod 400 x 4 FP64 took 18.6 -> 5.7, Couette 4 x 200 FP64 28.6 -> 5.9 and FP32
-// 4.8 -> 2.6, slip Couette 100 x 5 FP64 29.4 -> 5.7 and FP32 12.0 -> 3.0.
+// Sod 400 x 4 FP64 took 18.6 -> 5.7, Couette 4 x 200 FP64 28.6 -> 5.8 and FP32
+// 4.8 -> 2.5, slip Couette 100 x 5 FP64 29.4 -> 5.9 and FP32 12.0 -> 3.1.
 template <typename R>
 bool use_split(const Layout& L, int version) {
   const bool wall = has_side(L, BC_WALL), diffuse = has_side(L, BC_DIFFUSE);
